@@ -159,6 +159,17 @@ xct_status xct_project(xct_plan_t plan, const float* x, float* y, int32_t S,
                        void* stream);
 
 /*
+ * xct_project_rows -- xct_project with every ray's sum taken in the order of
+ * its stored entries, as the products inside xct_cgls take it (xct_project
+ * and xct_backproject of 16-bit slices sum blocks of 16 columns on the
+ * tensor cores first: the same FP32 accumulation in another order).  For
+ * costs that are reported in FP64: the data term of the differentiable
+ * reconstruction is computed from it.
+ */
+xct_status xct_project_rows(xct_plan_t plan, const float* x, float* y, int32_t S,
+                            void* stream);
+
+/*
  * xct_backproject -- x = A^T y with the stored transpose (Sec. III-B: the
  * same kernel serves projection and back projection).  y: [S][M][N_d],
  * x: [S][n][n] (overwritten).  Exact adjoint of xct_project in F32 storage.

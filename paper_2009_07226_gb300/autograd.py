@@ -50,7 +50,9 @@ class DataFit(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, x, y, plan):
-        q = plan.project(x.contiguous())
+        x = x.contiguous()
+        q = torch.empty((x.shape[0], plan.m, plan.nd), dtype=torch.float32, device=x.device)
+        xct.xct_project_rows(plan.handle, x, q, x.shape[0])
         r = torch.empty_like(q)
         val = torch.empty((), dtype=torch.float64, device=x.device)
         xct.xct_datafit(q, y.contiguous(), r, q[0].numel(), q.shape[0], val)

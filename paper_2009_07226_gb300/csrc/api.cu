@@ -470,6 +470,7 @@ xct_status apply_pipelined(Plan& p, bool transposed, const float* in, float* out
   const int32_t* in_inv = transposed ? p.ray_inv : p.pix_inv;
   const int32_t* out_inv = transposed ? p.pix_inv : p.ray_inv;
   const int64_t nin = L.ncols, nout = L.nrows;
+  const OctLayout* oct = octets_for(p, transposed, st);
   Arena ar(s);
   float *Xn[2] = {nullptr, nullptr}, *Yn[2] = {nullptr, nullptr}, *Xi[2], *Yi[2];
   uint32_t* mx[2];
@@ -478,8 +479,10 @@ xct_status apply_pipelined(Plan& p, bool transposed, const float* in, float* out
   for (int b = 0; b < 2; ++b) {
     if (in_host) XCT_TRY(ar.get(&Xn[b], (size_t)nin * st));
     if (out_host) XCT_TRY(ar.get(&Yn[b], (size_t)nout * st));
-    XCT_TRY(ar.get(&Xi[b], (size_t)nin * st));
-    XCT_TRY(ar.get(&Yi[b], (size_t)nout * st));
+    if (!oct) {
+      XCT_TRY(ar.get(&Xi[b], (size_t)nin * st));
+      XCT_TRY(ar.get(&Yi[b], (size_t)nout * st));
+    }
     XCT_TRY(ar.get(&mx[b], (size_t)st));
     if (stages16(p.storage)) XCT_TRY(ar.get(&h16[b], (size_t)nin * st));
   }
@@ -507,23 +510,30 @@ xct_status apply_pipelined(Plan& p, bool transposed, const float* in, float* out
       XCT_TRY_CUDA(cudaStreamWaitEvent(s, ev_in[b].e, 0));
       xin = Xn[b];
     }
-    XCT_TRY_CUDA(cudaMemsetAsync(mx[b], 0, sizeof(uint32_t) * st, s));
-    XCT_TRY(to_internal(xin, Xi[b], in_inv, nin, St, st, 1, mx[b], s));
-    if (in_host) XCT_TRY_CUDA(cudaEventRecord(ev_used[b].e, s));
-    SpmmArgs a{&L, Xi[b], Yi[b], st, 1, p.storage, p.mat_scale_exp, mx[b], nullptr, h16[b], work,
-               p.err};
-    XCT_TRY(spmm(a, s));
     float* yout = out + (size_t)t * st * nout;
+    float* ydev = out_host ? Yn[b] : yout;
+    if (oct) {
+      const OctProduct a{xin, ydev, St, st, in_inv, out_inv, p.mat_scale_exp, mx[b], h16[b], work, p.err};
+      XCT_TRY(oct_stage(*oct, a, p.storage, s));
+      if (in_host) XCT_TRY_CUDA(cudaEventRecord(ev_used[b].e, s));
+      if (out_host && t >= 2) XCT_TRY_CUDA(cudaStreamWaitEvent(s, ev_d2h[b].e, 0));
+      XCT_TRY(oct_run(*oct, a, p.storage, s));
+    } else {
+      XCT_TRY_CUDA(cudaMemsetAsync(mx[b], 0, sizeof(uint32_t) * st, s));
+      XCT_TRY(to_internal(xin, Xi[b], in_inv, nin, St, st, 1, mx[b], s));
+      if (in_host) XCT_TRY_CUDA(cudaEventRecord(ev_used[b].e, s));
+      SpmmArgs a{&L, Xi[b], Yi[b], st, 1, p.storage, p.mat_scale_exp, mx[b], nullptr, h16[b], work,
+                 p.err};
+      XCT_TRY(spmm(a, s));
+      if (out_host && t >= 2) XCT_TRY_CUDA(cudaStreamWaitEvent(s, ev_d2h[b].e, 0));
+      XCT_TRY(to_natural(Yi[b], ydev, out_inv, nout, St, st, 1, s));
+    }
     if (out_host) {
-      if (t >= 2) XCT_TRY_CUDA(cudaStreamWaitEvent(s, ev_d2h[b].e, 0));
-      XCT_TRY(to_natural(Yi[b], Yn[b], out_inv, nout, St, st, 1, s));
       XCT_TRY_CUDA(cudaEventRecord(ev_out[b].e, s));
       XCT_TRY_CUDA(cudaStreamWaitEvent(cout.s, ev_out[b].e, 0));
       XCT_TRY_CUDA(cudaMemcpyAsync(yout, Yn[b], sizeof(float) * St * nout, cudaMemcpyDeviceToHost,
                                    cout.s));
       XCT_TRY_CUDA(cudaEventRecord(ev_d2h[b].e, cout.s));
-    } else {
-      XCT_TRY(to_natural(Yi[b], yout, out_inv, nout, St, st, 1, s));
     }
   }
   XCT_TRY_CUDA(cudaStreamSynchronize(cin.s));
@@ -531,8 +541,10 @@ xct_status apply_pipelined(Plan& p, bool transposed, const float* in, float* out
   return check_kernel_flag(p, s);
 }
 
+// rows: on the row layouts, each row summed in its own order (the products
+// of costs that are reported in FP64)
 xct_status apply_impl(Plan& p, bool transposed, const float* in, float* out, int32_t S,
-                      cudaStream_t s) {
+                      cudaStream_t s, bool rows = false) {
   const Layout& L = transposed ? p.lat : p.la;
   const int32_t* in_inv = transposed ? p.ray_inv : p.pix_inv;
   const int32_t* out_inv = transposed ? p.pix_inv : p.ray_inv;
@@ -541,26 +553,32 @@ xct_status apply_impl(Plan& p, bool transposed, const float* in, float* out, int
   const int ntiles = (S + st - 1) / st;
   const int S_pad = st * ntiles;
   const bool in_host = is_host_pointer(in), out_host = is_host_pointer(out);
-  if ((in_host || out_host) && ntiles > 1)
+  if ((in_host || out_host) && ntiles > 1 && !rows)
     return apply_pipelined(p, transposed, in, out, S, st, ntiles, in_host, out_host, s);
+  const OctLayout* oct = rows ? nullptr : octets_for(p, transposed, st);
   Arena ar(s);
   DevView iv, ov;
   XCT_TRY(device_view(in, (size_t)S * nin, true, ar, s, iv));
   XCT_TRY(device_view(out, (size_t)S * nout, false, ar, s, ov));
-  float *Xi, *Yi;
   uint32_t* mx;
-  XCT_TRY(ar.get(&Xi, (size_t)nin * S_pad));
-  XCT_TRY(ar.get(&Yi, (size_t)nout * S_pad));
   XCT_TRY(ar.get(&mx, (size_t)S_pad));
   uint16_t* h16 = nullptr;
   if (stages16(p.storage)) XCT_TRY(ar.get(&h16, (size_t)nin * S_pad));
   int* work;
   XCT_TRY(ar.get(&work, 1));
-  XCT_TRY_CUDA(cudaMemsetAsync(mx, 0, sizeof(uint32_t) * S_pad, s));
-  XCT_TRY(to_internal(iv.dev, Xi, in_inv, nin, S, st, ntiles, mx, s));
-  SpmmArgs a{&L, Xi, Yi, st, ntiles, p.storage, p.mat_scale_exp, mx, nullptr, h16, work, p.err};
-  XCT_TRY(spmm(a, s));
-  XCT_TRY(to_natural(Yi, ov.dev, out_inv, nout, S, st, ntiles, s));
+  if (oct) {
+    XCT_TRY(oct_product(*oct, OctProduct{iv.dev, ov.dev, S, st, in_inv, out_inv, p.mat_scale_exp, mx, h16, work,
+                                         p.err}, p.storage, s));
+  } else {
+    float *Xi, *Yi;
+    XCT_TRY(ar.get(&Xi, (size_t)nin * S_pad));
+    XCT_TRY(ar.get(&Yi, (size_t)nout * S_pad));
+    XCT_TRY_CUDA(cudaMemsetAsync(mx, 0, sizeof(uint32_t) * S_pad, s));
+    XCT_TRY(to_internal(iv.dev, Xi, in_inv, nin, S, st, ntiles, mx, s));
+    SpmmArgs a{&L, Xi, Yi, st, ntiles, p.storage, p.mat_scale_exp, mx, nullptr, h16, work, p.err};
+    XCT_TRY(spmm(a, s));
+    XCT_TRY(to_natural(Yi, ov.dev, out_inv, nout, S, st, ntiles, s));
+  }
   if (ov.host) {
     XCT_TRY_CUDA(cudaMemcpyAsync(out, ov.dev, sizeof(float) * S * nout, cudaMemcpyDeviceToHost, s));
     return check_kernel_flag(p, s);
@@ -695,6 +713,17 @@ xct_status xct_backproject(xct_plan_t plan, const float* y, float* x, int32_t S,
   }
   if (S == 0) return XCT_OK;
   return apply_impl(*plan, true, y, x, S, static_cast<cudaStream_t>(stream));
+}
+
+xct_status xct_project_rows(xct_plan_t plan, const float* x, float* y, int32_t S, void* stream) {
+  Trace trace_("xct_project_rows");
+  XCT_TRY(check_plan(plan));
+  if (S < 0 || ((!x || !y) && S > 0)) {
+    set_error("bad arguments (S = %d)", S);
+    return XCT_ERR_INVALID;
+  }
+  if (S == 0) return XCT_OK;
+  return apply_impl(*plan, false, x, y, S, static_cast<cudaStream_t>(stream), true);
 }
 
 xct_status xct_cgls(xct_plan_t plan, const float* y, float* x, int32_t S, int32_t iters,

@@ -485,13 +485,6 @@ __device__ int64_t block_sum64(int64_t v, int64_t* red) {
   return t;
 }
 
-struct CsrView {
-  const int64_t* rowptr;
-  const int32_t* col;
-  const double* val;
-  int64_t nrows, ncols;
-};
-
 __device__ void block_col_range(const CsrView& m, int64_t e0, int64_t e1, int32_t* lo_hi) {
   int32_t lo = INT32_MAX, hi = -1;
   for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
@@ -1711,6 +1704,26 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
         mem.release();
         out = Layout{};
       }
+    }
+  }
+
+  // octet layouts for products between natural vectors of 16-bit slices;
+  // where device memory runs out or a stage does not fit, those products use
+  // the layouts above
+  if (stages16(p.storage)) {
+    for (int which = 0; which < 2; ++which) {
+      Arena mem(s);
+      OctLayout& out = which == 0 ? p.oa : p.oat;
+      bool fits = false;
+      const xct_status st = build_oct_layout(which == 0 ? ma : mt, p.storage, which == 0, out, mem, &fits, s);
+      if (st == XCT_ERR_OOM || (st == XCT_OK && !fits)) {
+        mem.release();
+        out = OctLayout{};
+        continue;
+      }
+      XCT_TRY(st);
+      mem.move_to(keep);
+      (which == 0 ? p.la : p.lat).oct = &out;
     }
   }
 

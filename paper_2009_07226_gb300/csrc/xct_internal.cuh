@@ -152,6 +152,62 @@ inline int64_t stage_desc_bytes(int64_t run_stride) {
   return (int64_t)sizeof(StageDescHead) + kQuads * 16 + 8 * run_stride;
 }
 
+// Octet layout of one matrix for products of 16-bit slices on the tensor
+// cores (spmm_mma.cu, built by octet_layout.cu).  A block is kOctRows
+// consecutive rows; its input footprint is a list of aligned groups of 8
+// columns, cut into stages of at most `cap` staged rows, a staged row's
+// position being congruent to its column mod 8.  A block's rows form octets
+// of 8 rows (for A 2 bins x 4 angles, for A^T 4 x 2 pixels of a tile), and
+// an octet's entries in a stage form dense chunks: 16 columns (the distinct
+// columns of the octet, 16 at a time) by 8 rows of 16-bit values.
+//
+// Chunk bytes: a stage's chunks are stored octet after octet as
+// [chunk][lane][8 bytes] values (256 bytes a chunk: lane 4 n + t holds rows
+// n of columns 2t, 2t + 1, 2t + 8, 2t + 9, the B fragment of an
+// mma.m16n8k16), then [chunk][16] positions of 2 bytes.  Within a chunk the
+// columns 0-7 and 8-15 have positions that are distinct mod 8 where the
+// counts allow, so that the 8 row reads of one ldmatrix phase fall in
+// distinct banks.  Unused columns carry value 0 and repeat a used position.
+constexpr int kOctRows = 128;
+constexpr int kOcts = kOctRows / 8;
+// Row of a 64-row group at place p (octet p / 8) of the octet order.  A full
+// tile of rays is numbered bin * 8 + angle: an octet takes 2 bins x 4 angles,
+// the bin fastest; a full tile of pixels (2 x 2 groups) in its own order.
+__host__ __device__ __forceinline__ int oct_row(int p, int angle_rows) {
+  if (!angle_rows) return p;
+  return (p & 48) | (p & 8) >> 1 | (p & 6) >> 1 | (p & 1) << 3;
+}
+constexpr int kChunkBytes = 256 + 32;
+// first stage capacity tried (projection of 64 slices at 512^2 x 768: 0.701
+// ms with 384, 0.708 with 256, 16 slices 0.352 and 0.443: the stage's fixed
+// costs; two buffers of 512 do not fit)
+constexpr int kOctCap = 384;
+// A stage's descriptor: this head, the first chunk of every octet (kOcts + 1
+// numbers), padded to 16 bytes, then the runs of its staged rows as (first
+// column, first position) pairs and closing pairs (-1, positions).
+struct __align__(16) OctStageHead {
+  int64_t c0;          // first chunk of the stage
+  uint32_t nch;        // chunks of the stage
+  uint16_t np;         // staged rows copied (columns past the matrix left out)
+  uint16_t nr;         // run-list pairs, closing pair included
+  uint16_t ofs[kOcts + 1];
+};
+
+struct OctLayout {
+  int64_t nrows = 0, ncols = 0;
+  int32_t nblocks = 0;
+  int32_t cap = 0;             // staged rows of a stage, a multiple of 64
+  int32_t angle_rows = 0;      // 1: rows are rays (see oct_row)
+  int64_t nstages = 0, nchunks = 0;
+  int64_t emax = 0;            // chunks of the largest stage
+  int64_t* blk_stage = nullptr;   // [nblocks + 1]
+  uint2* chunks = nullptr;        // [nstages] first chunk, chunks
+  unsigned char* desc = nullptr;  // [nstages] descriptors of desc_bytes each
+  int64_t desc_bytes = 0;
+  unsigned char* ent = nullptr;   // chunk bytes, stage after stage
+  int64_t bytes = 0;
+};
+
 struct Layout {
   int64_t nrows = 0, ncols = 0;
   int32_t nblocks = 0;
@@ -187,6 +243,8 @@ struct Layout {
   // runs are those of the plain layout, its segments and 8-byte slots its own)
   const Layout* paired = nullptr;
   bool pair = false;
+  // the octet layout of the same matrix (see octets_for)
+  const OctLayout* oct = nullptr;
   int64_t gathers = 0;         // paired: distinct columns of the pairs over all stages
                                // (the staged-row reads of one tile, padding aside)
   int64_t bytes = 0;
@@ -257,6 +315,7 @@ struct Plan {
   Layout la, lat;
   Layout law, latw;              // wide-stage layouts (XCT_PLAN_FEW_SLICES)
   Layout lap, latp;              // paired layouts (XCT_PLAN_PAIRED_ROWS)
+  OctLayout oa, oat;             // octet layouts (16-bit slices)
   int32_t mat_scale_exp = 0;     // k: stored value = RN(l * 2^k)
   int* err = nullptr;            // device flag: a bounded wait in a kernel ran out
   // kept FP64 matrices (ordered ids), only with XCT_PLAN_KEEP_F64
@@ -266,6 +325,31 @@ struct Plan {
   xct_stats stats{};
   std::map<int, int> tile_choice;  // measured slice-tile width per slice count
 };
+
+// a matrix in ordered ids, as traced or transposed (FP64 values)
+struct CsrView {
+  const int64_t* rowptr;
+  const int32_t* col;
+  const double* val;
+  int64_t nrows, ncols;
+};
+// the octet layout of a matrix (octet_layout.cu); *fits is false, and
+// nothing kept, when its stage buffers would not fit a product's CTA
+xct_status build_oct_layout(const CsrView& m, xct_dtype storage, bool angle_rows, OctLayout& L,
+                            Arena& keep, bool* fits, cudaStream_t s);
+
+// The octet layout that a product of the plan's matrix (or its transpose)
+// between natural vectors runs on, for slice tiles of st; nullptr: it runs on
+// the row layouts (FP32 slices; 8-slice tiles of a plan with wide-stage
+// layouts, which stream fewer bytes: 0.20 - 0.23 ms against 0.34 at 512^2 x
+// 768; a matrix whose octet layout did not fit).  Products inside solves, and
+// those whose FP64 cost is reported, stay on the row layouts: they keep each
+// row's order of summation, so that logged residual norms and costs do not
+// move.
+inline const OctLayout* octets_for(const Plan& p, bool transposed, int st) {
+  const Layout& L = transposed ? p.lat : p.la;
+  return stages16(p.storage) && !(st == 8 && L.wide) ? L.oct : nullptr;
+}
 
 // plan building (plan.cu)
 xct_status build_plan(Plan& p, cudaStream_t s);
@@ -318,6 +402,12 @@ inline SpmmArgs on_product_layout(SpmmArgs a) {
   else if (a.L->paired && stages16(a.storage) && a.st * 2 == kEntryRowBytes) a.L = a.L->paired;
   return a;
 }
+// byte offset of the 16-byte chunk c of a 16-bit staged row of `rowb` bytes
+// as octet products read it: chunks are permuted within the row by the
+// row's id (congruent to its staged position mod 8), so that the same chunk
+// of 8 rows of distinct ids mod 8 lies in 8 distinct 16-byte bank groups
+__host__ __device__ constexpr int oct_swz_shift(int rowb) { return rowb >= 128 ? 0 : rowb == 64 ? 1 : 2; }
+__host__ __device__ constexpr int oct_swz_mask(int rowb) { return rowb >= 128 ? 7 : rowb / 16 - 1; }
 xct_status spmm(const SpmmArgs& a, cudaStream_t s);   // = spmm_stage + spmm_run
 // 16-bit storage: the normalised 16-bit copy of the input (no-op for FP32)
 xct_status spmm_stage(const SpmmArgs& a, cudaStream_t s);
@@ -332,6 +422,24 @@ xct_status spmm_pipe(const SpmmArgs& a, cudaStream_t s);
 constexpr int kMaxPipeProducts = 8;
 bool spmm_pipe_multi_applies(const SpmmArgs* list, int count);
 xct_status spmm_pipe_multi(const SpmmArgs* list, int count, cudaStream_t s);
+// A product of 16-bit slices on an octet layout (spmm_mma.cu), between
+// natural-layout device vectors.
+struct OctProduct {
+  const float* x;          // [S][ncols]
+  float* y;                // [S][nrows]
+  int S, st;               // slices, slices per tile
+  const int32_t *col_inv, *row_inv;   // ordered -> natural ids
+  int mat_scale_exp;
+  uint32_t* in_max;        // scratch [ntiles * st]
+  uint16_t* staged;        // scratch [ntiles][ncols][st]
+  int* work;               // scratch: a work counter
+  int* err;                // device flag set to 1 if a bounded wait ran out
+};
+// = oct_stage (reads x: maxima, staged rows) + oct_run (writes y)
+xct_status oct_product(const OctLayout& L, const OctProduct& p, xct_dtype storage, cudaStream_t s);
+xct_status oct_stage(const OctLayout& L, const OctProduct& p, xct_dtype storage, cudaStream_t s);
+xct_status oct_run(const OctLayout& L, const OctProduct& p, xct_dtype storage, cudaStream_t s);
+bool oct_stage_fits(int cap, int64_t emax, int64_t desc_bytes);
 // number of per-slice partial sums spmm() writes for dot_partial (per slice):
 // one per block of rows
 int spmm_dot_count(const SpmmArgs& a);

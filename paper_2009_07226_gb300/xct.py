@@ -79,6 +79,8 @@ _SIGNATURES = [
     ("xct_free", None, [ctypes.c_void_p]),
     ("xct_project", ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                    ctypes.c_int32, ctypes.c_void_p]),
+    ("xct_project_rows", ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
+                                        ctypes.c_int32, ctypes.c_void_p]),
     ("xct_backproject", ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                        ctypes.c_int32, ctypes.c_void_p]),
     ("xct_cgls", ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32,
@@ -213,6 +215,11 @@ def xct_free(plan: int) -> None:
 
 def xct_project(plan: int, x, y, S: int, stream=None) -> None:
     _check(lib().xct_project(plan, _ptr(x), _ptr(y), S, _stream(stream)))
+
+
+def xct_project_rows(plan: int, x, y, S: int, stream=None) -> None:
+    """y = A x, each ray summed in the order of its entries (as in a solve)."""
+    _check(lib().xct_project_rows(plan, _ptr(x), _ptr(y), S, _stream(stream)))
 
 
 def xct_project_noalloc(plan: int, x, y, S: int, stream=None) -> None:
