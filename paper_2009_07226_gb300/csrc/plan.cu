@@ -13,6 +13,8 @@
 
 #include <algorithm>
 #include <chrono>
+#include <cmath>
+#include <type_traits>
 
 #include "xct_internal.cuh"
 
@@ -162,105 +164,123 @@ __device__ __forceinline__ double plane_alpha(int i, double half, double p, doub
   return ddiv(dsub(dsub((double)i, half), p), d);
 }
 
+// num / d correctly rounded, from y = RN(1 / d): the quotient num * y is
+// corrected twice by its exact remainder.  The first correction leaves it
+// within an ulp, from where the second rounds correctly (Markstein's theorem
+// on division with fused multiply-add, 1990).  Five dependent FP64
+// instructions, where the general division takes some thirty.  y = 0 (a
+// direction component so small or large that the steps could leave the FP64
+// range) takes the general division.
+__device__ __forceinline__ double quotient(double num, double d, double y) {
+  if (__double_as_longlong(y) == 0) return ddiv(num, d);
+  double q = dmul(num, y);
+  q = __fma_rn(__fma_rn(-q, d, num), y, q);
+  return __fma_rn(__fma_rn(-q, d, num), y, q);
+}
+
+__device__ __forceinline__ double reciprocal_for_quotient(double d) {
+  return fabs(d) > 1e-100 && fabs(d) < 1e100 ? __drcp_rn(d) : 0.0;
+}
+
 // Crossings of one axis strictly inside (amin, amax), in ascending alpha:
-// planes first..last stepping by step (empty when count == 0).  alpha(i) is
-// monotone in i, so each bound is found by bisection on the exact predicate.
+// planes first..last stepping by step (empty when count == 0).
 struct AxisWalk {
   int i, step, left;
 };
 
-__device__ AxisWalk axis_walk(const Ray& r, double p, double d) {
+// alpha(i) is monotone in i, so each bound follows from a guess (the line's
+// coordinate where the ray enters or leaves) moved until the exact predicate
+// changes there.
+__device__ AxisWalk axis_walk(const Ray& r, double p, double d, double y) {
   AxisWalk w{0, 1, 0};
   const int n = r.n;
   if (d == 0.0 || n < 2) return w;
+  auto alpha = [&](int i) { return quotient(dsub(dsub((double)i, r.half), p), d, y); };
+  auto guess = [&](double a) {
+    const double g = floor(dadd(dadd(p, dmul(a, d)), r.half));
+    return g < 0.0 ? 0 : (g > (double)n ? n : (int)g);
+  };
+  // planes 1 .. n - 1 with alpha > amin and alpha < amax
+  int lo, hi;   // first and last of them
   if (d > 0.0) {
-    // first i with alpha(i) > amin  (predicate false..true)
-    int lo = 1, hi = n;  // hi = none
-    while (lo < hi) {
-      int mid = (lo + hi) >> 1;
-      if (plane_alpha(mid, r.half, p, d) > r.amin) hi = mid; else lo = mid + 1;
-    }
-    int first = lo;
-    // last i with alpha(i) < amax (predicate true..false)
-    lo = 0;
-    hi = n - 1;  // lo = none
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (plane_alpha(mid, r.half, p, d) < r.amax) lo = mid; else hi = mid - 1;
-    }
-    int last = lo;
-    if (first <= n - 1 && last >= 1 && first <= last) {
-      w.i = first;
-      w.step = 1;
-      w.left = last - first + 1;
-    }
+    lo = max(1, guess(r.amin) + 1);
+    while (lo > 1 && alpha(lo - 1) > r.amin) --lo;
+    while (lo < n && !(alpha(lo) > r.amin)) ++lo;
+    hi = min(n - 1, guess(r.amax));
+    while (hi < n - 1 && alpha(hi + 1) < r.amax) ++hi;
+    while (hi > 0 && !(alpha(hi) < r.amax)) --hi;
   } else {
-    // alpha decreasing in i: ascending alpha walks i downwards
-    // last i with alpha(i) > amin (predicate true..false)
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-      int mid = (lo + hi + 1) >> 1;
-      if (plane_alpha(mid, r.half, p, d) > r.amin) lo = mid; else hi = mid - 1;
-    }
-    int top = lo;
-    // first i with alpha(i) < amax (predicate false..true)
-    lo = 1;
-    hi = n;
-    while (lo < hi) {
-      int mid = (lo + hi) >> 1;
-      if (plane_alpha(mid, r.half, p, d) < r.amax) hi = mid; else lo = mid + 1;
-    }
-    int bottom = lo;
-    if (top >= 1 && bottom <= n - 1 && bottom <= top) {
-      w.i = top;
-      w.step = -1;
-      w.left = top - bottom + 1;
-    }
+    hi = min(n - 1, guess(r.amin));
+    while (hi < n - 1 && alpha(hi + 1) > r.amin) ++hi;
+    while (hi > 0 && !(alpha(hi) > r.amin)) --hi;
+    lo = max(1, guess(r.amax) + 1);
+    while (lo > 1 && alpha(lo - 1) < r.amax) --lo;
+    while (lo < n && !(alpha(lo) < r.amax)) ++lo;
+  }
+  if (lo <= n - 1 && hi >= 1 && lo <= hi) {
+    w.step = d > 0.0 ? 1 : -1;
+    w.i = d > 0.0 ? lo : hi;
+    w.left = hi - lo + 1;
   }
   return w;
 }
 
-// Walk the merged crossings; sink(pixel, length) for each kept segment.
+// Walk the merged crossings; sink(pixel, length) for each kept segment.  FP64
+// instructions run at a 64th of the FP32 rate here, so a step has about a
+// dozen: the next crossing of the axis just crossed, the length, and
+// comparisons.  A segment's pixel is the one of its midpoint; the planes
+// crossed give it directly where the midpoint lies clear of the grid lines
+// (half the segment's extent along each axis against 1e-10, far above the
+// midpoint's rounding error), else it is computed.
 template <class Sink>
 __device__ void trace(const Ray& r, Sink& sink) {
-  AxisWalk wx = axis_walk(r, r.px, r.dx);
-  AxisWalk wy = axis_walk(r, r.py, r.dy);
-  double ax = wx.left ? plane_alpha(wx.i, r.half, r.px, r.dx) : 0.0;
-  double ay = wy.left ? plane_alpha(wy.i, r.half, r.py, r.dy) : 0.0;
+  const double yx = reciprocal_for_quotient(r.dx), yy = reciprocal_for_quotient(r.dy);
+  AxisWalk wx = axis_walk(r, r.px, r.dx, yx);
+  AxisWalk wy = axis_walk(r, r.py, r.dy, yy);
+  // plane coordinates of the next crossings (exact in FP64), as i - half
+  double cx = dsub((double)wx.i, r.half), cy = dsub((double)wy.i, r.half);
+  const double sx = (double)wx.step, sy = (double)wy.step;
+  double ax = wx.left ? quotient(dsub(cx, r.px), r.dx, yx) : INFINITY;
+  double ay = wy.left ? quotient(dsub(cy, r.py), r.dy, yy) : INFINITY;
   double cur = r.amin;
   const int n = r.n;
-  while (true) {
-    double nxt;
-    int which;
-    if (wx.left && (!wy.left || ax <= ay)) {
-      nxt = ax;
-      which = 0;
-    } else if (wy.left) {
-      nxt = ay;
-      which = 1;
-    } else {
-      nxt = r.amax;
-      which = 2;
-    }
-    double len = dsub(nxt, cur);
+  // the pixel before the next crossings, known along an axis that is crossed
+  int ix = wx.step > 0 ? wx.i - 1 : wx.i, iy = wy.step > 0 ? wy.i - 1 : wy.i;
+  const float clear = wx.left && wy.left ? fminf(fabsf((float)r.dx), fabsf((float)r.dy)) : 0.0f;
+  const int steps = wx.left + wy.left;
+  for (int k = 0;; ++k) {
+    const bool last = k == steps;
+    const bool isx = !last && wx.left && (!wy.left || ax <= ay);
+    const double nxt = last ? r.amax : (isx ? ax : ay);
+    const double len = dsub(nxt, cur);
     if (len >= r.min_seg) {
-      double mid = dmul(dadd(cur, nxt), 0.5);
-      double x = dadd(r.px, dmul(mid, r.dx));
-      double y = dadd(r.py, dmul(mid, r.dy));
-      int ix = (int)floor(dadd(x, r.half));
-      int iy = (int)floor(dadd(y, r.half));
-      ix = ix < 0 ? 0 : (ix > n - 1 ? n - 1 : ix);
-      iy = iy < 0 ? 0 : (iy > n - 1 ? n - 1 : iy);
-      sink(iy * n + ix, len);
+      int jx = ix, jy = iy;
+      if (!((float)len * clear > 2e-10f)) {
+        const double mid = dmul(dadd(cur, nxt), 0.5);
+        const double x = dadd(r.px, dmul(mid, r.dx));
+        const double y = dadd(r.py, dmul(mid, r.dy));
+        jx = (int)floor(dadd(x, r.half));
+        jy = (int)floor(dadd(y, r.half));
+      }
+      jx = jx < 0 ? 0 : (jx > n - 1 ? n - 1 : jx);
+      jy = jy < 0 ? 0 : (jy > n - 1 ? n - 1 : jy);
+      sink(jy * n + jx, len);
     }
+    if (last) break;
     cur = nxt;
-    if (which == 2) break;
-    if (which == 0) {
-      wx.i += wx.step;
-      if (--wx.left) ax = plane_alpha(wx.i, r.half, r.px, r.dx);
+    // the axis just crossed moves on (one division for both cases)
+    const double c = dadd(isx ? cx : cy, isx ? sx : sy);
+    const double a = quotient(dsub(c, isx ? r.px : r.py), isx ? r.dx : r.dy, isx ? yx : yy);
+    if (isx) {
+      cx = c;
+      ax = a;
+      ix += wx.step;
+      --wx.left;
     } else {
-      wy.i += wy.step;
-      if (--wy.left) ay = plane_alpha(wy.i, r.half, r.py, r.dy);
+      cy = c;
+      ay = a;
+      iy += wy.step;
+      --wy.left;
     }
   }
 }
@@ -316,34 +336,162 @@ __global__ void siddon_fill_kernel(GeomDev g, const int32_t* ray_inv, const int3
   if (setup_row(g, ray_inv[h], r)) trace(r, sink);
 }
 
-// Matrix-free projection (no stored A): each thread traces one ray with the
-// plan builder's arithmetic and accumulates RN32(length) * x[s][pixel] in
-// FP32 for kMfSlices slices per pass, retracing the ray for the next ones.
+// Matrix-free projection (no stored A): each thread traces one ray and
+// accumulates RN32(length) * x[s][pixel] in FP32.
+//
+// FP64 instructions would bound it (a trace step takes a dozen even so), so
+// the walk itself runs in 64-bit integers: crossing parameters in units of
+// 2^-bits with |alpha| < 2^60 units, each axis's crossings a constant step
+// apart, the first crossing and the step from FP64.  The parameters drift by
+// at most half a unit a crossing (n * 2^-bits / 2: 1e-13 at n = 512, 5e-10 at
+// the largest grid), far below a length's rounding to FP32.  Rays nearly
+// along an axis (a component below 1e-4, where a line on a grid line could
+// take either side) and directions that are not unit vectors are traced as
+// the plan builder traces them.
+// The slices are interleaved in tiles first, so a step reads one contiguous
+// piece of kMfSlices slices instead of as many distant words.
+// 256^2 x 384, 24 slices: 61.7 -> 0.83 ms a call (three tiles of 8; before,
+// every tile walked in FP64 and read each slice on its own).
 constexpr int kMfSlices = 8;
 
-struct ProjSink {
-  const float* x;      // natural [S][npix]
-  int64_t npix;
-  int s0, ns;
-  float acc[kMfSlices];
-  __device__ void operator()(int pix, double len) {
-    const float l = (float)len;
+struct FxRay {
+  long long cur, ax, ay, sx, sy, amax;   // start, next crossings, steps, end
+  int ix, iy, nx, ny;                    // pixel, crossings left with the direction's sign
+};
+constexpr int kFxMiss = INT32_MIN, kFxExact = INT32_MIN + 1;   // FxRay::nx
+
+__global__ void __launch_bounds__(128) fx_setup_kernel(GeomDev g, int64_t nray, int bits, FxRay* out) {
+  const int64_t ray = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (ray >= nray) return;
+  FxRay f{};
+  Ray r;
+  if (!setup_row(g, (int32_t)ray, r)) {
+    f.nx = kFxMiss;
+  } else if (fabs(r.dx) < 1e-4 || fabs(r.dy) < 1e-4 || fabs(r.dx * r.dx + r.dy * r.dy - 1.0) > 1e-6) {
+    f.nx = kFxExact;
+  } else {
+    const double yx = reciprocal_for_quotient(r.dx), yy = reciprocal_for_quotient(r.dy);
+    const AxisWalk wx = axis_walk(r, r.px, r.dx, yx), wy = axis_walk(r, r.py, r.dy, yy);
+    const double unit = (double)(1ll << bits), most = (double)(1ll << 61);
+    auto fixed = [&](double a) { return __double2ll_rn(a * unit); };
+    f.cur = fixed(r.amin);
+    f.amax = fixed(r.amax);
+    f.ax = wx.left ? fixed(plane_alpha(wx.i, r.half, r.px, r.dx)) : 0;
+    f.ay = wy.left ? fixed(plane_alpha(wy.i, r.half, r.py, r.dy)) : 0;
+    f.sx = __double2ll_rn(fmin(fabs(yx) * unit, most));
+    f.sy = __double2ll_rn(fmin(fabs(yy) * unit, most));
+    // before its next crossing an axis is in the pixel on the near side of
+    // the plane; without crossings, in the one of the chord's midpoint
+    const double mid = 0.5 * (r.amin + r.amax);
+    auto side = [&](const AxisWalk& w, double p, double d) {
+      const int c = w.left ? (w.step > 0 ? w.i - 1 : w.i) : (int)floor(p + mid * d + r.half);
+      return c < 0 ? 0 : (c > r.n - 1 ? r.n - 1 : c);
+    };
+    f.ix = side(wx, r.px, r.dx);
+    f.iy = side(wy, r.py, r.dy);
+    f.nx = r.dx > 0.0 ? wx.left : -wx.left;
+    f.ny = r.dy > 0.0 ? wy.left : -wy.left;
+  }
+  out[ray] = f;
+}
+
+// natural [S][npix] -> [tiles][npix][NS] (slices past S are zero)
+template <int NS>
+__global__ void __launch_bounds__(256) interleave_kernel(const float* __restrict__ x, float* __restrict__ out,
+                                                         int64_t npix, int S) {
+  const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (p >= npix) return;
+  const int s0 = blockIdx.y * NS;
+  float v[NS];
 #pragma unroll
-    for (int k = 0; k < kMfSlices; ++k)
-      if (k < ns) acc[k] = fmaf(l, __ldg(x + (size_t)(s0 + k) * npix + pix), acc[k]);
+  for (int k = 0; k < NS; ++k) v[k] = s0 + k < S ? x[(size_t)(s0 + k) * npix + p] : 0.0f;
+  float* o = out + ((size_t)blockIdx.y * npix + p) * NS;
+#pragma unroll
+  for (int k = 0; k < NS; ++k) o[k] = v[k];
+}
+
+template <int NS>
+struct Piece {
+  float v[NS];
+  __device__ __forceinline__ void load(const float* p) {
+    if constexpr (NS % 4 == 0) {
+#pragma unroll
+      for (int k = 0; k < NS; k += 4) {
+        const float4 t = __ldg(reinterpret_cast<const float4*>(p + k));
+        v[k] = t.x; v[k + 1] = t.y; v[k + 2] = t.z; v[k + 3] = t.w;
+      }
+    } else if constexpr (NS == 2) {
+      const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+      v[0] = t.x; v[1] = t.y;
+    } else {
+      v[0] = __ldg(p);
+    }
   }
 };
 
-__global__ void matfree_project_kernel(GeomDev g, const float* x, float* y, int S, int64_t nray) {
+template <int NS>
+struct ProjSink {
+  const float* x;      // [npix][NS]
+  float acc[NS];
+  __device__ void operator()(int pix, double len) {
+    const float l = (float)len;
+    Piece<NS> t;
+    t.load(x + (size_t)pix * NS);
+#pragma unroll
+    for (int k = 0; k < NS; ++k) acc[k] = fmaf(l, t.v[k], acc[k]);
+  }
+};
+
+template <int NS>
+__global__ void __launch_bounds__(128) matfree_project_kernel(GeomDev g, const FxRay* __restrict__ rays, int bits,
+                                                              long long min_len, const float* __restrict__ xt,
+                                                              float* __restrict__ y, int S, int64_t nray) {
   const int64_t ray = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (ray >= nray) return;
-  Ray r;
-  const bool hit = setup_row(g, (int32_t)ray, r);
-  for (int s0 = 0; s0 < S; s0 += kMfSlices) {
-    ProjSink sink{x, (int64_t)g.n * g.n, s0, min(kMfSlices, S - s0), {}};
-    if (hit) trace(r, sink);
-    for (int k = 0; k < sink.ns; ++k) y[(size_t)(s0 + k) * nray + ray] = sink.acc[k];
+  const int n = g.n, s0 = blockIdx.y * NS;
+  ProjSink<NS> sink{xt + (size_t)blockIdx.y * n * n * NS, {}};
+  const FxRay f = rays[ray];
+  if (f.nx == kFxExact) {
+    Ray r;
+    if (setup_row(g, (int32_t)ray, r)) trace(r, sink);
+  } else if (f.nx != kFxMiss) {
+    constexpr long long kNone = INT64_MAX;
+    const float unit = __int_as_float((127 - bits) << 23);   // 2^-bits
+    const int dx = f.nx > 0 ? 1 : -1, dy = f.ny > 0 ? n : -n;
+    int nx = abs(f.nx), ny = abs(f.ny), pix = f.iy * n + f.ix;
+    long long cur = f.cur, ax = nx ? f.ax : kNone, ay = ny ? f.ay : kNone;
+    // each segment's slices are loaded while the one before is added
+    float lp = 0.0f;
+    Piece<NS> tp{};
+    for (int left = nx + ny; left >= 0; --left) {
+      const bool isx = ax <= ay;
+      const long long nxt = left == 0 ? f.amax : (isx ? ax : ay), len = nxt - cur;
+      const bool kept = len >= min_len;
+      Piece<NS> t{};
+      if (kept) t.load(sink.x + (size_t)pix * NS);
+      if (lp > 0.0f) {
+#pragma unroll
+        for (int k = 0; k < NS; ++k) sink.acc[k] = fmaf(lp, tp.v[k], sink.acc[k]);
+      }
+      lp = kept ? __ll2float_rn(len) * unit : 0.0f;
+      tp = t;
+      cur = nxt;
+      if (isx) {
+        pix += dx;
+        ax = --nx > 0 ? ax + f.sx : kNone;
+      } else {
+        pix += dy;
+        ay = --ny > 0 ? ay + f.sy : kNone;
+      }
+    }
+    if (lp > 0.0f) {
+#pragma unroll
+      for (int k = 0; k < NS; ++k) sink.acc[k] = fmaf(lp, tp.v[k], sink.acc[k]);
+    }
   }
+#pragma unroll
+  for (int k = 0; k < NS; ++k)
+    if (s0 + k < S) y[(size_t)(s0 + k) * nray + ray] = sink.acc[k];
 }
 
 // ---------------------------------------------------------------------------
@@ -1554,10 +1702,41 @@ xct_status matfree_project(const Plan& p, const double* cs_dev, const float* x, 
                            cudaStream_t s) {
   const xct_geometry& g = p.g;
   GeomDev gd{g.n, g.n_angles, g.n_det, g.det_spacing, g.det_offset, g.min_seg, cs_dev};
-  matfree_project_kernel<<<grid_for(p.nray, 128), 128, 0, s>>>(gd, x, y, S, p.nray);
+  // crossing parameters stay within the grid's half diagonal and a little:
+  // |alpha| < 2^k with 2^k >= 1.5 n
+  int k = 1;
+  while ((1ll << k) < (3ll * g.n + 1) / 2) ++k;
+  const int bits = 60 - k;
+  const double least = std::min(g.min_seg * (double)(1ll << bits), (double)(1ll << 62));
+  const long long min_len = std::max(1ll, (long long)std::llround(least));
+  Arena tmp(s);
+  FxRay* rays;
+  XCT_TRY(tmp.get(&rays, p.nray));
+  fx_setup_kernel<<<grid_for(p.nray, 128), 128, 0, s>>>(gd, p.nray, bits, rays);
   count_launch();
-  XCT_TRY_CUDA(cudaGetLastError());
-  return XCT_OK;
+  auto run = [&](auto ns) -> xct_status {
+    constexpr int NS = decltype(ns)::value;
+    const int tiles = (S + NS - 1) / NS;
+    const float* xt = x;
+    if (NS > 1) {
+      float* t;
+      XCT_TRY(tmp.get(&t, (size_t)p.npix * tiles * NS));
+      for (int t0 = 0; t0 < tiles; t0 += 65535)
+        interleave_kernel<NS><<<dim3(grid_for(p.npix, 256), std::min(tiles - t0, 65535)), 256, 0, s>>>(
+            x + (size_t)t0 * NS * p.npix, t + (size_t)t0 * NS * p.npix, p.npix, S - t0 * NS);
+      xt = t;
+    }
+    for (int t0 = 0; t0 < tiles; t0 += 65535)
+      matfree_project_kernel<NS><<<dim3(grid_for(p.nray, 128), std::min(tiles - t0, 65535)), 128, 0, s>>>(
+          gd, rays, bits, min_len, xt + (size_t)t0 * NS * p.npix, y + (size_t)t0 * NS * p.nray, S - t0 * NS, p.nray);
+    count_launch(NS > 1 ? 2 : 1);
+    XCT_TRY_CUDA(cudaGetLastError());
+    return XCT_OK;
+  };
+  if (S == 1) return run(std::integral_constant<int, 1>());
+  if (S == 2) return run(std::integral_constant<int, 2>());
+  if (S <= 4) return run(std::integral_constant<int, 4>());
+  return run(std::integral_constant<int, kMfSlices>());
 }
 
 xct_status build_plan(Plan& p, cudaStream_t s) {
