@@ -507,9 +507,11 @@ __global__ void col_count_kernel(const int32_t* col, int64_t nnz, int32_t* ccoun
 __global__ void transpose_fill_kernel(const int64_t* rowptr, const int32_t* col, const double* val,
                                       int64_t nrow, unsigned long long* cursor, int32_t* trow,
                                       double* tval) {
-  int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  // a warp per row
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (r >= nrow) return;
-  for (int64_t e = rowptr[r]; e < rowptr[r + 1]; ++e) {
+  const int64_t e1 = rowptr[r + 1];
+  for (int64_t e = rowptr[r] + (threadIdx.x & 31); e < e1; e += 32) {
     unsigned long long p = atomicAdd(&cursor[col[e]], 1ull);
     trow[p] = (int32_t)r;
     tval[p] = val[e];
@@ -588,7 +590,7 @@ xct_status transpose(const int64_t* rowptr, const int32_t* col, const double* va
   XCT_TRY(exclusive_scan_i32(ccount, colptr, ncol, s));
   XCT_TRY_CUDA(cudaMemcpyAsync(cursor, colptr, sizeof(int64_t) * ncol, cudaMemcpyDeviceToDevice, s));
   if (nnz > 0) {
-    transpose_fill_kernel<<<grid_for(nrow, 128), 128, 0, s>>>(rowptr, col, val, nrow, cursor, trow, tval);
+    transpose_fill_kernel<<<grid_for(32 * nrow, 128), 128, 0, s>>>(rowptr, col, val, nrow, cursor, trow, tval);
     max_count_kernel<<<grid_for(ncol, 256, 1024), 256, 0, s>>>(ccount, ncol, dmax);
     count_launch(2);
     int32_t hmax = 0;
@@ -684,29 +686,22 @@ __device__ void mark_window(const CsrView& m, int64_t e0, int64_t e1, int64_t w0
       const int i = threadIdx.x * kPer + k;
       const uint64_t lo = i > 0 ? bm[i - 1] : 0u, hi = i + 1 < kWinWords ? bm[i + 1] : 0u;
       const uint32_t mid = bm[i];
-      uint32_t f = 0;
       // an empty word lies inside a gap of at least 32 > `gap` columns, and a
       // full word has nothing to fill
       if (mid == 0u || mid == 0xffffffffu) {
         fill[k] = 0u;
         continue;
       }
-      for (int j = 0; j < 32; ++j) {
-        if ((mid >> j) & 1u) continue;
-        // nearest set bits below and above bit j of mid in the 96-bit view
-        int dl = 0, dr = 0;
-        for (int d = 1; d <= gap; ++d) {
-          const int q = 32 + j - d;
-          const uint32_t w = q < 32 ? (uint32_t)lo : mid;
-          if ((w >> (q & 31)) & 1u) { dl = d; break; }
-        }
-        for (int d = 1; d <= gap; ++d) {
-          const int q = 32 + j + d;
-          const uint32_t w = q < 64 ? mid : (uint32_t)hi;
-          if ((w >> (q & 31)) & 1u) { dr = d; break; }
-        }
-        if (dl > 0 && dr > 0 && dl + dr - 1 <= gap) f |= 1u << j;
+      // a column is filled when set ones lie dl below and dr above it with
+      // dl + dr - 1 <= gap: for each dl, the ones dl below against the union
+      // of the ones 1 .. gap + 1 - dl above
+      const uint64_t below = (uint64_t)mid << 32 | lo, above = hi << 32 | mid;
+      uint32_t f = 0, up = 0;
+      for (int dl = gap; dl >= 1; --dl) {
+        up |= (uint32_t)(above >> (gap + 1 - dl));
+        f |= (uint32_t)(below >> (32 - dl)) & up;
       }
+      f &= ~mid;
       fill[k] = f;
     }
     __syncthreads();
@@ -838,58 +833,86 @@ __global__ void stage_np_kernel(const int64_t* blk_stage, const int64_t* fp_size
 // Contiguous runs of each stage's staged rows, for one bulk copy per run:
 // pairs (first row id, first position in the stage), then a closing pair
 // (-1, rows of the stage) repeated to an even count (16-byte aligned lists).
-// One thread per block walks the block's stages.
-__global__ void run_count_kernel(const int64_t* blk_stage, const int64_t* fp_off,
-                                 const int64_t* fp_size, const int32_t* pix, int32_t nblocks,
-                                 int32_t cap, int64_t* nrun, unsigned long long* rmax) {
-  int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b >= nblocks) return;
-  for (int64_t s = blk_stage[b]; s < blk_stage[b + 1]; ++s) {
+// A warp takes a block's stages one after another, 32 staged rows at a time.
+constexpr int kRunWarps = 4;
+__global__ void __launch_bounds__(32 * kRunWarps) run_count_kernel(
+    const int64_t* blk_stage, const int64_t* fp_off, const int64_t* fp_size, const int32_t* pix,
+    int32_t nblocks, int32_t cap, int64_t* nrun, unsigned long long* rmax) {
+  const int b = blockIdx.x, lane = threadIdx.x & 31;
+  for (int64_t s = blk_stage[b] + (threadIdx.x >> 5); s < blk_stage[b + 1]; s += kRunWarps) {
     const int64_t k = s - blk_stage[b];
     const int64_t p0 = fp_off[b] + k * cap;
-    const int64_t n = min((int64_t)cap, fp_size[b] - k * cap);
+    const int n = (int)min((int64_t)cap, fp_size[b] - k * cap);
     int64_t r = 0;
-    for (int64_t i = 0; i < n; ++i)
-      if (i == 0 || pix[p0 + i] != pix[p0 + i - 1] + 1) ++r;
-    nrun[s] = (r + 2) & ~(int64_t)1;
-    atomicMax(rmax, (unsigned long long)nrun[s]);
+    for (int i = lane; i < n; i += 32) r += i == 0 || pix[p0 + i] != pix[p0 + i - 1] + 1;
+    for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (lane == 0) {
+      nrun[s] = (r + 2) & ~(int64_t)1;
+      atomicMax(rmax, (unsigned long long)nrun[s]);
+    }
   }
 }
 
-__global__ void run_fill_kernel(const int64_t* blk_stage, const int64_t* fp_off,
-                                const int64_t* fp_size, const int32_t* pix, int32_t nblocks,
-                                int32_t cap, const int64_t* run_off, int2* runs) {
-  int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b >= nblocks) return;
-  for (int64_t s = blk_stage[b]; s < blk_stage[b + 1]; ++s) {
+__global__ void __launch_bounds__(32 * kRunWarps) run_fill_kernel(
+    const int64_t* blk_stage, const int64_t* fp_off, const int64_t* fp_size, const int32_t* pix,
+    int32_t nblocks, int32_t cap, const int64_t* run_off, int2* runs) {
+  const int b = blockIdx.x, lane = threadIdx.x & 31;
+  for (int64_t s = blk_stage[b] + (threadIdx.x >> 5); s < blk_stage[b + 1]; s += kRunWarps) {
     const int64_t k = s - blk_stage[b];
     const int64_t p0 = fp_off[b] + k * cap;
     const int n = (int)min((int64_t)cap, fp_size[b] - k * cap);
     int64_t o = run_off[s];
-    for (int i = 0; i < n; ++i)
-      if (i == 0 || pix[p0 + i] != pix[p0 + i - 1] + 1) runs[o++] = make_int2(pix[p0 + i], i);
-    for (; o < run_off[s + 1]; ++o) runs[o] = make_int2(-1, n);
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      const bool starts = i < n && (i == 0 || pix[p0 + i] != pix[p0 + i - 1] + 1);
+      const uint32_t m = __ballot_sync(0xffffffffu, starts);
+      if (starts) runs[o + __popc(m & ((1u << lane) - 1u))] = make_int2(pix[p0 + i], i);
+      o += __popc(m);
+    }
+    for (o += lane; o < run_off[s + 1]; o += 32) runs[o] = make_int2(-1, n);
+  }
+}
+
+// A warp walks one row, 32 entries at a time, and calls f(entry, stage - s0,
+// position in the stage, index among the row's entries of that stage in
+// their order) for the entries of stages [s0, s0 + kStageChunk); cnt receives
+// the row's entries per stage.
+constexpr int kRowThreads = 512;
+template <class F>
+__device__ __forceinline__ void for_row_entries(const CsrView& m, const int32_t* epos, int64_t row, int32_t cap,
+                                                int64_t s0, uint16_t* cnt, F f) {
+  const int lane = threadIdx.x & 31;
+  for (int k = lane; k < kStageChunk; k += 32) cnt[k] = 0;
+  __syncwarp();
+  if (row >= m.nrows) return;
+  const int64_t e0 = m.rowptr[row], e1 = m.rowptr[row + 1];
+  for (int64_t eb = e0; eb < e1; eb += 32) {
+    const int64_t e = eb + lane;
+    const int32_t p = e < e1 ? epos[e] : 0;
+    int64_t st = e < e1 ? p / cap - s0 : -1;
+    if (st < 0 || st >= kStageChunk) st = -1;
+    const uint32_t same = __match_any_sync(0xffffffffu, (int)st);
+    const int before = __popc(same & ((1u << lane) - 1u));
+    const int k = st >= 0 ? cnt[st] + before : 0;
+    __syncwarp();
+    if (st >= 0 && before == 0) cnt[st] = (uint16_t)(k + __popc(same));
+    __syncwarp();
+    if (st >= 0) f(e, (int)st, p % cap, k);
   }
 }
 
 // per (stage, quad): the 4 row counts and the padded slot count (the
 // quad's longest row rounded up to `per_row` entries, for each of 4 rows)
-__global__ void __launch_bounds__(kRowsPerBlock) seg_count_kernel(CsrView m, const int32_t* epos,
-                                                                  const int64_t* blk_stage,
-                                                                  int32_t cap, int32_t per_row,
-                                                                  Seg* seg, int64_t* slots) {
+__global__ void __launch_bounds__(kRowThreads) seg_count_kernel(CsrView m, const int32_t* epos,
+                                                                const int64_t* blk_stage,
+                                                                int32_t cap, int32_t per_row,
+                                                                Seg* seg, int64_t* slots) {
   __shared__ uint16_t cnt[kRowsPerBlock][kStageChunk + 2];  // counts <= capacity
-  const int b = blockIdx.x;
+  const int b = blockIdx.x, warp = threadIdx.x >> 5;
   const int64_t sb = blk_stage[b], ns = blk_stage[b + 1] - sb;
-  const int64_t row = (int64_t)b * kRowsPerBlock + threadIdx.x;
-  const bool has = row < m.nrows;
-  const int64_t e0 = has ? m.rowptr[row] : 0, e1 = has ? m.rowptr[row + 1] : 0;
   for (int64_t s0 = 0; s0 < ns; s0 += kStageChunk) {
-    for (int k = 0; k < kStageChunk; ++k) cnt[threadIdx.x][k] = 0;
-    for (int64_t e = e0; e < e1; ++e) {
-      int64_t st = epos[e] / cap - s0;
-      if (st >= 0 && st < kStageChunk) cnt[threadIdx.x][st] = (uint16_t)(cnt[threadIdx.x][st] + 1);
-    }
+    for (int r = warp; r < kRowsPerBlock; r += kRowThreads / 32)
+      for_row_entries(m, epos, (int64_t)b * kRowsPerBlock + r, cap, s0, cnt[r], [](int64_t, int, int, int) {});
     __syncthreads();
     const int64_t nchunk = min((int64_t)kStageChunk, ns - s0);
     for (int64_t i = threadIdx.x; i < nchunk * kQuads; i += blockDim.x) {
@@ -981,29 +1004,21 @@ __device__ __forceinline__ void pack_entry(void* ent, int64_t slot, uint32_t loc
 }
 
 template <int KIND>
-__global__ void __launch_bounds__(kRowsPerBlock) fill_entries_kernel(CsrView m, const int32_t* epos,
-                                                                     const int64_t* blk_stage,
-                                                                     int32_t cap, const Seg* seg,
-                                                                     void* ent, uint32_t unit) {
-  __shared__ uint16_t cnt[kRowsPerBlock][kStageChunk + 2];  // counts <= capacity
-  const int b = blockIdx.x;
+__global__ void __launch_bounds__(kRowThreads) fill_entries_kernel(CsrView m, const int32_t* epos,
+                                                                   const int64_t* blk_stage,
+                                                                   int32_t cap, const Seg* seg,
+                                                                   void* ent, uint32_t unit) {
+  __shared__ uint16_t cnt[kRowThreads / 32][kStageChunk];  // counts <= capacity
+  const int b = blockIdx.x, warp = threadIdx.x >> 5;
   const int64_t sb = blk_stage[b], ns = blk_stage[b + 1] - sb;
-  const int64_t row = (int64_t)b * kRowsPerBlock + threadIdx.x;
-  if (row >= m.nrows) return;
-  const int q = threadIdx.x / 4, g = threadIdx.x % 4;
-  const int64_t e0 = m.rowptr[row], e1 = m.rowptr[row + 1];
-  for (int64_t s0 = 0; s0 < ns; s0 += kStageChunk) {
-    for (int k = 0; k < kStageChunk; ++k) cnt[threadIdx.x][k] = 0;
-    for (int64_t e = e0; e < e1; ++e) {
-      int32_t p = epos[e];
-      int64_t st = p / cap - s0;
-      if (st < 0 || st >= kStageChunk) continue;
-      int32_t k = cnt[threadIdx.x][st];
-      cnt[threadIdx.x][st] = (uint16_t)(k + 1);
-      int64_t slot = seg[(sb + s0 + st) * kQuads + q].off + (k >> 2) * 16 + g * 4 + (k & 3);
-      pack_entry<KIND>(ent, slot, (uint32_t)(p % cap), m.val[e], unit);
-    }
-  }
+  for (int64_t s0 = 0; s0 < ns; s0 += kStageChunk)
+    for (int r = warp; r < kRowsPerBlock; r += kRowThreads / 32)
+      for_row_entries(m, epos, (int64_t)b * kRowsPerBlock + r, cap, s0, cnt[warp],
+                      [&](int64_t e, int st, int p, int k) {
+                        const int64_t slot = seg[(sb + s0 + st) * kQuads + r / 4].off + (k >> 2) * 16 +
+                                             (r % 4) * 4 + (k & 3);
+                        pack_entry<KIND>(ent, slot, (uint32_t)p, m.val[e], unit);
+                      });
 }
 
 // Entry order of a wide-stage layout (16-byte staged rows, 16-bit entries).
@@ -1212,7 +1227,7 @@ xct_status build_layout(const CsrView& m, int64_t nnz, xct_dtype storage, int32_
     XCT_TRY(own.get(&L.stage_run, L.nstages + 1));
     XCT_TRY_CUDA(cudaMemsetAsync(rmax, 0, sizeof(unsigned long long), s));
     if (nb > 0) {
-      run_count_kernel<<<grid_for(nb, 128), 128, 0, s>>>(L.blk_stage, fp_off, fp_size, L.pix, nb, cap,
+      run_count_kernel<<<nb, 32 * kRunWarps, 0, s>>>(L.blk_stage, fp_off, fp_size, L.pix, nb, cap,
                                                          nrun, rmax);
       count_launch();
     }
@@ -1227,14 +1242,14 @@ xct_status build_layout(const CsrView& m, int64_t nnz, xct_dtype storage, int32_
     L.run_max = (int64_t)rmax_h;
     XCT_TRY(own.get(&L.runs, nruns));
     if (nb > 0) {
-      run_fill_kernel<<<grid_for(nb, 128), 128, 0, s>>>(L.blk_stage, fp_off, fp_size, L.pix, nb, cap,
+      run_fill_kernel<<<nb, 32 * kRunWarps, 0, s>>>(L.blk_stage, fp_off, fp_size, L.pix, nb, cap,
                                                         L.stage_run, L.runs);
       count_launch();
     }
   }
   if (nb > 0) {
     // wide-stage layouts: groups of 4 chunks per row (see wide_order_kernel)
-    seg_count_kernel<<<nb, kRowsPerBlock, 0, s>>>(m, epos, L.blk_stage, cap,
+    seg_count_kernel<<<nb, kRowThreads, 0, s>>>(m, epos, L.blk_stage, cap,
                                                   unit == kWideRowBytes ? 16 : 4, L.seg, slots);
     count_launch();
   }
@@ -1272,13 +1287,13 @@ xct_status build_layout(const CsrView& m, int64_t nnz, xct_dtype storage, int32_
   count_launch();
   if (nb > 0) {
     if (storage == XCT_F32)
-      fill_entries_kernel<0><<<nb, kRowsPerBlock, 0, s>>>(m, epos, L.blk_stage, cap, L.seg, L.ent,
+      fill_entries_kernel<0><<<nb, kRowThreads, 0, s>>>(m, epos, L.blk_stage, cap, L.seg, L.ent,
                                                             (uint32_t)unit);
     else if (half_values(storage))
-      fill_entries_kernel<1><<<nb, kRowsPerBlock, 0, s>>>(m, epos, L.blk_stage, cap, L.seg, L.ent,
+      fill_entries_kernel<1><<<nb, kRowThreads, 0, s>>>(m, epos, L.blk_stage, cap, L.seg, L.ent,
                                                             (uint32_t)unit);
     else
-      fill_entries_kernel<2><<<nb, kRowsPerBlock, 0, s>>>(m, epos, L.blk_stage, cap, L.seg, L.ent,
+      fill_entries_kernel<2><<<nb, kRowThreads, 0, s>>>(m, epos, L.blk_stage, cap, L.seg, L.ent,
                                                             (uint32_t)unit);
     count_launch();
   }
@@ -1405,14 +1420,16 @@ __global__ void pair_fill_kernel(const uint32_t* src, const Seg* seg, const Seg*
         return reg_b + (int64_t)(c / kPairUB) * 4 * kPairUB + (2 * p + e) * kPairUB + c % kPairUB;
       };
       int ns = 0, n0 = 0, n1 = 0;
+      int at = 0;   // the rows' orders mostly agree: the search starts after the last match
       for (int k = 0; k < c0; ++k) {
         const uint32_t e = src[pair_src_slot(sg, 2 * p, k)];
         const int q = pair_pos(e);
         if ((b1[q >> 5] >> (q & 31)) & 1u) {
           uint32_t f = 0u;
-          for (int j = 0; j < c1; ++j) {
+          for (int i = 0; i < c1; ++i) {
+            const int j = at + i < c1 ? at + i : at + i - c1;
             const uint32_t h = src[pair_src_slot(sg, 2 * p + 1, j)];
-            if ((h >> 16) == (e >> 16)) { f = h; break; }
+            if ((h >> 16) == (e >> 16)) { f = h; at = j + 1 < c1 ? j + 1 : 0; break; }
           }
           if (ns < ns_cap) {
             dst[2 * sa(ns)] = e;
