@@ -437,7 +437,7 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, bool angle_rows
   // stage capacity: the first at which two stage buffers of 128-byte rows
   // fit a CTA
   for (int cap = kOctCap; cap >= 64; cap = cap * 3 / 4 / 64 * 64) {
-    Arena own(s), part(s);
+    Arena own(s, true), part(s);
     L.cap = cap;
     const int gps = cap / 8;
     const int bm_smem = kOcts * kStageWindow * cap / 8;

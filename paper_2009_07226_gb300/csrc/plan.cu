@@ -1194,7 +1194,7 @@ xct_status build_layout(const CsrView& m, int64_t nnz, xct_dtype storage, int32_
   XCT_TRY_CUDA(cudaMemcpyAsync(&total_fp, fp_off + nb, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   XCT_TRY_CUDA(cudaStreamSynchronize(s));
   L.footprint = total_fp;
-  Arena own(s);
+  Arena own(s, true);
   XCT_TRY(own.get(&L.pix, total_fp + 4));   // padded lists, +4 for rounded copies
   XCT_TRY_CUDA(cudaMemsetAsync(L.pix, 0, sizeof(int32_t) * (total_fp + 4), s));
   XCT_TRY(own.get(&L.blk_stage, nb + 1));
@@ -1489,7 +1489,7 @@ xct_status build_paired_layout(const Layout& L, Layout& P, Arena& keep, cudaStre
   P.unit = kEntryRowBytes;
   P.pair = true;
   const int64_t nq = L.nstages * kQuads;
-  Arena tmp(s), own(s);
+  Arena tmp(s), own(s, true);
   int64_t *slots, *slot_off;
   unsigned int* bad;
   unsigned long long *emax, *gath;
@@ -1789,7 +1789,7 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   int32_t* cnt;
   int64_t* rowptr;
   XCT_TRY(tmp.get(&cnt, p.nray));
-  Arena f64(s);  // FP64 CSR / CSC, kept only with XCT_PLAN_KEEP_F64
+  Arena f64(s, (p.flags & XCT_PLAN_KEEP_F64) != 0);  // FP64 CSR / CSC, kept only with XCT_PLAN_KEEP_F64
   XCT_TRY(f64.get(&rowptr, p.nray + 1));
   siddon_count_kernel<<<grid_for(p.nray, 128), 128, 0, s>>>(gd, p.ray_inv, p.nray, cnt);
   count_launch();
@@ -1823,7 +1823,7 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   const int32_t cap0 = p.storage == XCT_F32 ? kPipeCap32 : kPipeCap16;
   auto fitted = [&](const CsrView& m, int32_t cap, Layout& L, Arena& mem) -> xct_status {
     for (int attempt = 0;; ++attempt) {
-      Arena lm(s);
+      Arena lm(s, true);
       Layout t;
       XCT_TRY(build_layout(m, p.nnz, p.storage, cap, t, lm, s, -1, kEntryRowBytes,
                            (p.flags & XCT_PLAN_NARROW_TILES) != 0));
@@ -1839,15 +1839,15 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
     const CsrView& m = which == 0 ? ma : mt;
     Layout& out = which == 0 ? p.la : p.lat;
     if (!(p.flags & XCT_PLAN_AUTOTUNE)) {
-      Arena mem(s);
+      Arena mem(s, true);
       XCT_TRY(fitted(m, cap0, out, mem));
       mem.move_to(keep);
       continue;
     }
     double best_ms = 1e300;
-    Arena best_mem(s);
+    Arena best_mem(s, true);
     for (int32_t cand : {cap0, (cap0 * 4 / 5) & ~3, (cap0 * 3 / 5) & ~3}) {
-      Arena mem(s);
+      Arena mem(s, true);
       Layout L;
       XCT_TRY(fitted(m, cand, L, mem));
       double ms = 0.0;
@@ -1867,7 +1867,7 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   // filled, offsets at 16 bytes per row; the entries stay in global memory
   if (p.flags & XCT_PLAN_FEW_SLICES) {
     for (int which = 0; which < 2; ++which) {
-      Arena mem(s);
+      Arena mem(s, true);
       Layout& out = which == 0 ? p.law : p.latw;
       XCT_TRY(build_layout(which == 0 ? ma : mt, p.nnz, p.storage, which == 0 ? kWideCapA : kWideCapAT, out, mem, s, kWideGap,
                            kWideRowBytes));
@@ -1884,7 +1884,7 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
     for (int which = 0; which < 2; ++which) {
       Layout& base = which == 0 ? p.la : p.lat;
       Layout& out = which == 0 ? p.lap : p.latp;
-      Arena mem(s);
+      Arena mem(s, true);
       XCT_TRY(build_paired_layout(base, out, mem, s));
       SpmmArgs probe{};
       probe.L = &out;
@@ -1908,7 +1908,7 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   // the layouts above
   if (stages16(p.storage)) {
     for (int which = 0; which < 2; ++which) {
-      Arena mem(s);
+      Arena mem(s, true);
       OctLayout& out = which == 0 ? p.oa : p.oat;
       bool fits = false;
       const xct_status st = build_oct_layout(which == 0 ? ma : mt, p.storage, which == 0, out, mem, &fits, s);

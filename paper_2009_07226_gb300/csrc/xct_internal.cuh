@@ -27,9 +27,13 @@ constexpr int kMaxDevices = 64;   // per-device caches of launch attributes
 extern std::atomic<int64_t> g_launches;
 inline void count_launch(int64_t k = 1) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
-// Device allocation through the configured allocator (cudaMallocAsync by
-// default).  Returns nullptr and sets the error message on failure.
-void* dalloc(size_t bytes, cudaStream_t s);
+// Device allocation through the configured allocator (by default
+// stream-ordered: working memory from the library's pool, memory that a plan
+// keeps from the device's default pool).  Returns nullptr and sets the error
+// message on failure.
+void* dalloc(size_t bytes, cudaStream_t s, bool keep = false);
+// a plan was made (1) or released (-1) on the device
+void scratch_plans(int device, int change);
 void dfree(void* p, size_t bytes, cudaStream_t s);
 
 // An NVTX range for the duration of an entry point (a no-op unless a
@@ -67,7 +71,8 @@ struct Arena {
   struct Item { void* p; size_t n; };
   std::vector<Item> items;
   cudaStream_t stream = nullptr;
-  explicit Arena(cudaStream_t s = nullptr) : stream(s) {}
+  bool keep = false;           // a plan's own memory
+  explicit Arena(cudaStream_t s = nullptr, bool keep_ = false) : stream(s), keep(keep_) {}
   Arena(const Arena&) = delete;
   Arena& operator=(const Arena&) = delete;
   ~Arena() { release(); }
@@ -75,7 +80,7 @@ struct Arena {
   xct_status get(T** out, size_t count) {
     size_t bytes = count * sizeof(T);
     if (bytes == 0) bytes = 256;
-    void* p = dalloc(bytes, stream);
+    void* p = dalloc(bytes, stream, keep);
     if (!p) { *out = nullptr; return XCT_ERR_OOM; }
     items.push_back({p, bytes});
     *out = static_cast<T*>(p);
@@ -321,7 +326,7 @@ struct Plan {
   // kept FP64 matrices (ordered ids), only with XCT_PLAN_KEEP_F64
   int64_t* a_rowptr = nullptr; int32_t* a_col = nullptr; double* a_val = nullptr;
   int64_t* t_rowptr = nullptr; int32_t* t_col = nullptr; double* t_val = nullptr;
-  Arena mem;                     // everything above lives here
+  Arena mem{nullptr, true};      // everything above lives here
   xct_stats stats{};
   std::map<int, int> tile_choice;  // measured slice-tile width per slice count
 };
