@@ -4,6 +4,8 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
+#include <initializer_list>
 #include <memory>
 #include <mutex>
 #include <vector>
@@ -254,6 +256,9 @@ xct_status enqueue_cgls(Plan& p, const float* yd, float* xd, int S, int st, int 
   const int S_pad = st * ntiles;
   const int64_t npix = p.npix, nray = p.nray;
   const int k = p.mat_scale_exp;
+  const int nv = vec_blocks(std::max(npix, nray), st);
+  int* work = B.work;          // a zeroed work counter for every product
+  XCT_TRY_CUDA(cudaMemsetAsync(B.work, 0, sizeof(int) * (2 * iters + 2), s));
   const SpmmArgs probe_at{&p.lat, B.R, B.Sv, st, ntiles, p.storage, k, B.sc.max_r, B.gpart,
                           B.h_ray, B.work, p.err};
   const int nb_at = spmm_dot_count(probe_at);
@@ -266,47 +271,48 @@ xct_status enqueue_cgls(Plan& p, const float* yd, float* xd, int S, int st, int 
     XCT_TRY_CUDA(cudaMemsetAsync(B.sc.max_r, 0, sizeof(uint32_t) * S_pad, s));
     XCT_TRY(to_internal(resume->r, B.R, p.ray_inv, nray, S, st, ntiles, B.sc.max_r, s));
     XCT_TRY_CUDA(cudaMemsetAsync(B.sc.max_r, 0, sizeof(uint32_t) * S_pad, s));
-    XCT_TRY(cgls_residual(B.R, nullptr, nray, st, ntiles, B.sc.max_r, B.rpart, s));
-    XCT_TRY(cgls_restore(resume->gamma, resume->active, S, B.rpart, B.sc, B.log, S_pad, s));
+    XCT_TRY(cgls_residual(B.R, nullptr, nray, st, ntiles, B.sc.max_r, B.rpart, nv, s));
+    XCT_TRY(cgls_restore(resume->gamma, resume->active, S, B.rpart, nv, B.sc, B.log, S_pad, s));
   } else {
     XCT_TRY_CUDA(cudaMemsetAsync(B.sc.max_r, 0, sizeof(uint32_t) * S_pad, s));
     XCT_TRY(to_internal(yd, B.R, p.ray_inv, nray, S, st, ntiles, B.sc.max_r, s));
     if (x0) {
       XCT_TRY_CUDA(cudaMemsetAsync(B.max_x, 0, sizeof(uint32_t) * S_pad, s));
       XCT_TRY(to_internal(xd, B.X, p.pix_inv, npix, S, st, ntiles, B.max_x, s));
-      SpmmArgs a{&p.la, B.X, B.Q, st, ntiles, p.storage, k, B.max_x, nullptr, B.h_pix, B.work, p.err};
+      SpmmArgs a{&p.la, B.X, B.Q, st, ntiles, p.storage, k, B.max_x, nullptr, B.h_pix, work++, p.err, true};
       XCT_TRY(spmm_timed(a, 0, tm, s));
       XCT_TRY_CUDA(cudaMemsetAsync(B.sc.max_r, 0, sizeof(uint32_t) * S_pad, s));
-      XCT_TRY(cgls_residual(B.R, B.Q, nray, st, ntiles, B.sc.max_r, B.rpart, s));
+      XCT_TRY(cgls_residual(B.R, B.Q, nray, st, ntiles, B.sc.max_r, B.rpart, nv, s));
     } else {
       XCT_TRY_CUDA(cudaMemsetAsync(B.X, 0, sizeof(float) * npix * S_pad, s));
-      XCT_TRY(cgls_residual(B.R, nullptr, nray, st, ntiles, B.sc.max_r, B.rpart, s));
+      XCT_TRY(cgls_residual(B.R, nullptr, nray, st, ntiles, B.sc.max_r, B.rpart, nv, s));
     }
     XCT_TRY_CUDA(cudaMemsetAsync(B.P, 0, sizeof(float) * npix * S_pad, s));
     {
-      SpmmArgs a{&p.lat, B.R, B.Sv, st, ntiles, p.storage, k, B.sc.max_r, B.gpart, B.h_ray, B.work, p.err};
+      SpmmArgs a{&p.lat, B.R, B.Sv, st, ntiles, p.storage, k, B.sc.max_r, B.gpart, B.h_ray, work++, p.err,
+                 true};
       XCT_TRY(spmm_timed(a, 1, tm, s));
     }
     if (tm) XCT_TRY(tm->begin(kPhScalar));
-    XCT_TRY(cgls_init_scalars(B.gpart, nb_at, B.rpart, B.sc, B.log, S_pad, s));
+    XCT_TRY(cgls_init_scalars(B.gpart, nb_at, B.rpart, nv, B.sc, B.log, S_pad, s));
     if (tm) XCT_TRY(tm->end(kPhScalar));
     if (tm) XCT_TRY(tm->begin(kPhVector));
     XCT_TRY(cgls_update_p(B.P, B.Sv, npix, st, ntiles, B.sc, s));
     if (tm) XCT_TRY(tm->end(kPhVector));
   }
   for (int it = 1; it <= iters; ++it) {
-    SpmmArgs ap{&p.la, B.P, B.Q, st, ntiles, p.storage, k, B.sc.max_p, B.dpart, B.h_pix, B.work, p.err};
+    SpmmArgs ap{&p.la, B.P, B.Q, st, ntiles, p.storage, k, B.sc.max_p, B.dpart, B.h_pix, work++, p.err, true};
     XCT_TRY(spmm_timed(ap, 0, tm, s));
     if (tm) XCT_TRY(tm->begin(kPhScalar));
     XCT_TRY(cgls_alpha(B.dpart, spmm_dot_count(ap), B.sc, S_pad, s));
     if (tm) XCT_TRY(tm->end(kPhScalar));
     if (tm) XCT_TRY(tm->begin(kPhVector));
-    XCT_TRY(cgls_update_xr(B.X, B.P, npix, B.R, B.Q, nray, st, ntiles, B.sc, B.rpart, s));
+    XCT_TRY(cgls_update_xr(B.X, B.P, npix, B.R, B.Q, nray, st, ntiles, B.sc, B.rpart, nv, s));
     if (tm) XCT_TRY(tm->end(kPhVector));
-    SpmmArgs at{&p.lat, B.R, B.Sv, st, ntiles, p.storage, k, B.sc.max_r, B.gpart, B.h_ray, B.work, p.err};
+    SpmmArgs at{&p.lat, B.R, B.Sv, st, ntiles, p.storage, k, B.sc.max_r, B.gpart, B.h_ray, work++, p.err, true};
     XCT_TRY(spmm_timed(at, 1, tm, s));
     if (tm) XCT_TRY(tm->begin(kPhScalar));
-    XCT_TRY(cgls_beta(B.gpart, nb_at, B.rpart, B.sc, B.log + (size_t)it * S_pad * 2, S_pad, s));
+    XCT_TRY(cgls_beta(B.gpart, nb_at, B.rpart, nv, B.sc, B.log + (size_t)it * S_pad * 2, S_pad, s));
     if (tm) XCT_TRY(tm->end(kPhScalar));
     if (tm) XCT_TRY(tm->begin(kPhVector));
     XCT_TRY(cgls_update_p(B.P, B.Sv, npix, st, ntiles, B.sc, s));
@@ -323,27 +329,12 @@ xct_status enqueue_cgls(Plan& p, const float* yd, float* xd, int S, int st, int 
   return XCT_OK;
 }
 
-struct StreamGuard {
-  cudaStream_t s = nullptr;
-  ~StreamGuard() {
-    if (s) cudaStreamDestroy(s);
-  }
-};
 struct EventGuard {
   cudaEvent_t e = nullptr;
   ~EventGuard() {
     if (e) cudaEventDestroy(e);
   }
 };
-struct GraphGuard {
-  cudaGraph_t g = nullptr;
-  cudaGraphExec_t x = nullptr;
-  ~GraphGuard() {
-    if (x) cudaGraphExecDestroy(x);
-    if (g) cudaGraphDestroy(g);
-  }
-};
-
 xct_status cgls_impl(Plan& p, const float* y, float* x, int32_t S, int32_t iters, uint32_t flags,
                      double* resid, void* state, cudaStream_t us) {
   const int st = pick_slices_per_tile(p.storage, S);
@@ -375,56 +366,33 @@ xct_status cgls_impl(Plan& p, const float* y, float* x, int32_t S, int32_t iters
   }
   const CglsState* resume_v = resume ? &st_view : nullptr;
   const CglsState* save_v = save ? &st_view : nullptr;
+  // working memory in four allocations (vectors, 16-bit copies, FP64 partial
+  // sums and scalars, words), each part on a 256-byte boundary
   CglsBufs B{};
-  XCT_TRY(ar.get(&B.X, (size_t)p.npix * S_pad));
-  XCT_TRY(ar.get(&B.P, (size_t)p.npix * S_pad));
-  XCT_TRY(ar.get(&B.Sv, (size_t)p.npix * S_pad));
-  XCT_TRY(ar.get(&B.R, (size_t)p.nray * S_pad));
-  XCT_TRY(ar.get(&B.Q, (size_t)p.nray * S_pad));
-  if (stages16(p.storage)) {
-    XCT_TRY(ar.get(&B.h_pix, (size_t)p.npix * S_pad));
-    XCT_TRY(ar.get(&B.h_ray, (size_t)p.nray * S_pad));
-  }
-  XCT_TRY(ar.get(&B.dpart, (size_t)S_pad * std::max(p.la.nblocks, 1)));
-  XCT_TRY(ar.get(&B.gpart, (size_t)S_pad * std::max(p.lat.nblocks, 1)));
-  XCT_TRY(ar.get(&B.work, 1));
-  XCT_TRY(ar.get(&B.rpart, (size_t)S_pad * kVecBlocks));
-  XCT_TRY(ar.get(&B.log, (size_t)(iters + 1) * S_pad * 2));
-  XCT_TRY(ar.get(&B.max_x, (size_t)S_pad));
-  XCT_TRY(ar.get(&B.sc.gamma, (size_t)S_pad));
-  XCT_TRY(ar.get(&B.sc.alpha, (size_t)S_pad));
-  XCT_TRY(ar.get(&B.sc.beta, (size_t)S_pad));
-  XCT_TRY(ar.get(&B.sc.active, (size_t)S_pad));
-  XCT_TRY(ar.get(&B.sc.active0, (size_t)S_pad));
-  XCT_TRY(ar.get(&B.sc.max_r, (size_t)S_pad));
-  XCT_TRY(ar.get(&B.sc.max_p, (size_t)S_pad));
+  auto carve = [&](std::initializer_list<std::pair<void**, size_t>> parts) -> xct_status {
+    size_t total = 0;
+    for (auto& q : parts) total += (q.second + 255) / 256 * 256;
+    unsigned char* base;
+    XCT_TRY(ar.get(&base, total));
+    for (auto& q : parts) {
+      *q.first = base;
+      base += (q.second + 255) / 256 * 256;
+    }
+    return XCT_OK;
+  };
+  const size_t fx = sizeof(float) * p.npix * S_pad, fr = sizeof(float) * p.nray * S_pad, d = sizeof(double) * S_pad,
+               w = sizeof(uint32_t) * S_pad;
+  XCT_TRY(carve({{(void**)&B.X, fx}, {(void**)&B.P, fx}, {(void**)&B.Sv, fx}, {(void**)&B.R, fr}, {(void**)&B.Q, fr}}));
+  if (stages16(p.storage)) XCT_TRY(carve({{(void**)&B.h_pix, fx / 2}, {(void**)&B.h_ray, fr / 2}}));
+  XCT_TRY(carve({{(void**)&B.dpart, d * std::max(p.la.nblocks, 1)}, {(void**)&B.gpart, d * std::max(p.lat.nblocks, 1)},
+                 {(void**)&B.rpart, d * kVecBlocks}, {(void**)&B.log, d * 2 * ((size_t)iters + 1)},
+                 {(void**)&B.sc.gamma, d}, {(void**)&B.sc.alpha, d}, {(void**)&B.sc.beta, d}}));
+  XCT_TRY(carve({{(void**)&B.work, sizeof(int) * (2 * (size_t)iters + 2)}, {(void**)&B.max_x, w},
+                 {(void**)&B.sc.active, w}, {(void**)&B.sc.active0, w}, {(void**)&B.sc.max_r, w},
+                 {(void**)&B.sc.max_p, w}}));
 
   const bool timing = (flags & XCT_CGLS_TIMING) != 0;
-  const bool graph = !(flags & (XCT_CGLS_NO_GRAPH | XCT_CGLS_TIMING));
-  if (graph) {
-    StreamGuard cs;
-    EventGuard e0, e1;
-    GraphGuard gg;
-    XCT_TRY_CUDA(cudaStreamCreateWithFlags(&cs.s, cudaStreamNonBlocking));
-    XCT_TRY_CUDA(cudaEventCreateWithFlags(&e0.e, cudaEventDisableTiming));
-    XCT_TRY_CUDA(cudaEventCreateWithFlags(&e1.e, cudaEventDisableTiming));
-    XCT_TRY_CUDA(cudaEventRecord(e0.e, us));
-    XCT_TRY_CUDA(cudaStreamWaitEvent(cs.s, e0.e, 0));
-    XCT_TRY_CUDA(cudaStreamBeginCapture(cs.s, cudaStreamCaptureModeThreadLocal));
-    xct_status st_enq = enqueue_cgls(p, yv.dev, xv.dev, S, st, ntiles, iters, x0, B, cs.s, nullptr,
-                                     resume_v, save_v, iters_before);
-    cudaError_t ec = cudaStreamEndCapture(cs.s, &gg.g);
-    if (st_enq != XCT_OK) return st_enq;
-    if (ec != cudaSuccess) {
-      set_error("graph capture failed: %s", cudaGetErrorString(ec));
-      return XCT_ERR_CUDA;
-    }
-    XCT_TRY_CUDA(cudaGraphInstantiate(&gg.x, gg.g, 0));
-    XCT_TRY_CUDA(cudaGraphLaunch(gg.x, cs.s));
-    XCT_TRY_CUDA(cudaEventRecord(e1.e, cs.s));
-    XCT_TRY_CUDA(cudaStreamWaitEvent(us, e1.e, 0));
-    XCT_TRY_CUDA(cudaStreamSynchronize(cs.s));
-  } else {
+  {
     PhaseTimer tm;
     tm.s = us;
     XCT_TRY(enqueue_cgls(p, yv.dev, xv.dev, S, st, ntiles, iters, x0, B, us,
@@ -979,24 +947,24 @@ xct_status xct_cgls_matfree(xct_plan_t plan, const float* y, float* x, int32_t S
   if (x0) {
     XCT_TRY_CUDA(cudaMemcpyAsync(X, xv.dev, sizeof(float) * npix * S, cudaMemcpyDeviceToDevice, s));
     XCT_TRY(matfree_project(p, cs_dev, X, Q, S, s));
-    XCT_TRY(cgls_residual(R, Q, nray, 1, S, sc.max_r, rpart, s));
+    XCT_TRY(cgls_residual(R, Q, nray, 1, S, sc.max_r, rpart, kVecBlocks, s));
   } else {
     XCT_TRY_CUDA(cudaMemsetAsync(X, 0, sizeof(float) * npix * S, s));
-    XCT_TRY(cgls_residual(R, nullptr, nray, 1, S, sc.max_r, rpart, s));
+    XCT_TRY(cgls_residual(R, nullptr, nray, 1, S, sc.max_r, rpart, kVecBlocks, s));
   }
   XCT_TRY(matfree_backproject(p, cs_dev, R, Sv, S, s));
-  XCT_TRY(cgls_residual(Sv, nullptr, npix, 1, S, sc.max_p, gpart, s));
-  XCT_TRY(cgls_init_scalars(gpart, kVecBlocks, rpart, sc, log, S, s));
+  XCT_TRY(cgls_residual(Sv, nullptr, npix, 1, S, sc.max_p, gpart, kVecBlocks, s));
+  XCT_TRY(cgls_init_scalars(gpart, kVecBlocks, rpart, kVecBlocks, sc, log, S, s));
   XCT_TRY_CUDA(cudaMemsetAsync(P, 0, sizeof(float) * npix * S, s));
   XCT_TRY(cgls_update_p(P, Sv, npix, 1, S, sc, s));
   for (int it = 1; it <= iters; ++it) {
     XCT_TRY(matfree_project(p, cs_dev, P, Q, S, s));
-    XCT_TRY(cgls_residual(Q, nullptr, nray, 1, S, sc.max_r, dpart, s));
+    XCT_TRY(cgls_residual(Q, nullptr, nray, 1, S, sc.max_r, dpart, kVecBlocks, s));
     XCT_TRY(cgls_alpha(dpart, kVecBlocks, sc, S, s));
-    XCT_TRY(cgls_update_xr(X, P, npix, R, Q, nray, 1, S, sc, rpart, s));
+    XCT_TRY(cgls_update_xr(X, P, npix, R, Q, nray, 1, S, sc, rpart, kVecBlocks, s));
     XCT_TRY(matfree_backproject(p, cs_dev, R, Sv, S, s));
-    XCT_TRY(cgls_residual(Sv, nullptr, npix, 1, S, sc.max_p, gpart, s));
-    XCT_TRY(cgls_beta(gpart, kVecBlocks, rpart, sc, log + (size_t)it * S * 2, S, s));
+    XCT_TRY(cgls_residual(Sv, nullptr, npix, 1, S, sc.max_p, gpart, kVecBlocks, s));
+    XCT_TRY(cgls_beta(gpart, kVecBlocks, rpart, kVecBlocks, sc, log + (size_t)it * S * 2, S, s));
     XCT_TRY(cgls_update_p(P, Sv, npix, 1, S, sc, s));
   }
   XCT_TRY_CUDA(cudaMemcpyAsync(xv.dev, X, sizeof(float) * npix * S, cudaMemcpyDeviceToDevice, s));

@@ -42,6 +42,7 @@ struct Group {
   double *dpart = nullptr, *gpart = nullptr, *rpart = nullptr, *log = nullptr;
   uint32_t* max_x = nullptr;
   CglsScalars sc{};
+  int nv() const { return vec_blocks(std::max(p->npix, p->nray), st); }
   SpmmArgs fwd() const {
     return SpmmArgs{&p->la, P, Q, st, ntiles, p->storage, p->mat_scale_exp, sc.max_p, dpart,
                     h_pix, nullptr, p->err};
@@ -196,16 +197,16 @@ xct_status enqueue_batch(std::vector<Group>& G, const xct_job* jobs, int iters, 
                  g.h_pix, work, p.err};
       XCT_TRY(spmm(a, s));
       XCT_TRY_CUDA(cudaMemsetAsync(g.sc.max_r, 0, sizeof(uint32_t) * g.S_pad, s));
-      XCT_TRY(cgls_residual(g.R, g.Q, p.nray, g.st, g.ntiles, g.sc.max_r, g.rpart, s));
+      XCT_TRY(cgls_residual(g.R, g.Q, p.nray, g.st, g.ntiles, g.sc.max_r, g.rpart, g.nv(), s));
     } else {
       XCT_TRY_CUDA(cudaMemsetAsync(g.X, 0, sizeof(float) * p.npix * g.S_pad, s));
-      XCT_TRY(cgls_residual(g.R, nullptr, p.nray, g.st, g.ntiles, g.sc.max_r, g.rpart, s));
+      XCT_TRY(cgls_residual(g.R, nullptr, p.nray, g.st, g.ntiles, g.sc.max_r, g.rpart, g.nv(), s));
     }
     XCT_TRY_CUDA(cudaMemsetAsync(g.P, 0, sizeof(float) * p.npix * g.S_pad, s));
   }
   XCT_TRY(product_phase(G, false, work, s));
   for (auto& g : G) {
-    XCT_TRY(cgls_init_scalars(g.gpart, spmm_dot_count(g.bwd()), g.rpart, g.sc, g.log, g.S_pad, s));
+    XCT_TRY(cgls_init_scalars(g.gpart, spmm_dot_count(g.bwd()), g.rpart, g.nv(), g.sc, g.log, g.S_pad, s));
     XCT_TRY(cgls_update_p(g.P, g.Sv, g.p->npix, g.st, g.ntiles, g.sc, s));
   }
   for (int it = 1; it <= iters; ++it) {
@@ -213,11 +214,11 @@ xct_status enqueue_batch(std::vector<Group>& G, const xct_job* jobs, int iters, 
     for (auto& g : G) {
       XCT_TRY(cgls_alpha(g.dpart, spmm_dot_count(g.fwd()), g.sc, g.S_pad, s));
       XCT_TRY(cgls_update_xr(g.X, g.P, g.p->npix, g.R, g.Q, g.p->nray, g.st, g.ntiles, g.sc,
-                             g.rpart, s));
+                             g.rpart, g.nv(), s));
     }
     XCT_TRY(product_phase(G, false, work, s));
     for (auto& g : G) {
-      XCT_TRY(cgls_beta(g.gpart, spmm_dot_count(g.bwd()), g.rpart, g.sc,
+      XCT_TRY(cgls_beta(g.gpart, spmm_dot_count(g.bwd()), g.rpart, g.nv(), g.sc,
                         g.log + (size_t)it * g.S_pad * 2, g.S_pad, s));
       XCT_TRY(cgls_update_p(g.P, g.Sv, g.p->npix, g.st, g.ntiles, g.sc, s));
     }

@@ -830,6 +830,14 @@ __global__ void stage_np_kernel(const int64_t* blk_stage, const int64_t* fp_size
     stage_np[s] = (int32_t)min((int64_t)cap, fp_size[b] - (s - blk_stage[b]) * cap);
 }
 
+__global__ void max_i64_kernel(const int64_t* v, int64_t n, unsigned long long* out) {
+  unsigned long long m = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    m = max(m, (unsigned long long)v[i]);
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
 // Contiguous runs of each stage's staged rows, for one bulk copy per run:
 // pairs (first row id, first position in the stage), then a closing pair
 // (-1, rows of the stage) repeated to an even count (16-byte aligned lists).
@@ -1223,23 +1231,26 @@ xct_status build_layout(const CsrView& m, int64_t nnz, xct_dtype storage, int32_
     int64_t* nrun;
     unsigned long long* rmax;
     XCT_TRY(tmp.get(&nrun, L.nstages));
-    XCT_TRY(tmp.get(&rmax, 1));
+    XCT_TRY(tmp.get(&rmax, 2));   // longest run list, largest footprint of a block
     XCT_TRY(own.get(&L.stage_run, L.nstages + 1));
-    XCT_TRY_CUDA(cudaMemsetAsync(rmax, 0, sizeof(unsigned long long), s));
+    XCT_TRY_CUDA(cudaMemsetAsync(rmax, 0, 2 * sizeof(unsigned long long), s));
     if (nb > 0) {
+      max_i64_kernel<<<grid_for(nb, 256, 152), 256, 0, s>>>(fp_size, nb, rmax + 1);
+      count_launch();
       run_count_kernel<<<nb, 32 * kRunWarps, 0, s>>>(L.blk_stage, fp_off, fp_size, L.pix, nb, cap,
                                                          nrun, rmax);
       count_launch();
     }
     XCT_TRY(exclusive_scan_i64(nrun, L.stage_run, L.nstages, s));
     int64_t nruns = 0;
-    unsigned long long rmax_h = 0;
+    unsigned long long rmax_h[2] = {0, 0};
     XCT_TRY_CUDA(cudaMemcpyAsync(&nruns, L.stage_run + L.nstages, sizeof(int64_t),
                                  cudaMemcpyDeviceToHost, s));
-    XCT_TRY_CUDA(cudaMemcpyAsync(&rmax_h, rmax, sizeof(rmax_h), cudaMemcpyDeviceToHost, s));
+    XCT_TRY_CUDA(cudaMemcpyAsync(rmax_h, rmax, sizeof(rmax_h), cudaMemcpyDeviceToHost, s));
     XCT_TRY_CUDA(cudaStreamSynchronize(s));
     L.nruns = nruns;
-    L.run_max = (int64_t)rmax_h;
+    L.run_max = (int64_t)rmax_h[0];
+    L.fp_max = (int64_t)rmax_h[1];
     XCT_TRY(own.get(&L.runs, nruns));
     if (nb > 0) {
       run_fill_kernel<<<nb, 32 * kRunWarps, 0, s>>>(L.blk_stage, fp_off, fp_size, L.pix, nb, cap,

@@ -476,6 +476,7 @@ xct_status spmm_run(const SpmmArgs& a0, cudaStream_t s) {
     set_error("unknown storage type");
     return XCT_ERR_INVALID;
   }
+  if (spmm_direct_applies(a)) return spmm_direct(a, s);
   if (spmm_pipe_applies(a)) return spmm_pipe(a, s);
   if (a.L->unit != kEntryRowBytes || a.L->pair) {
     set_error("wide-stage or paired layout without a fitting persistent product");

@@ -959,7 +959,7 @@ xct_status launch_pipe(const SpmmArgs* list, int count, cudaStream_t st) {
   XCT_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cur_dev));
   if (work == 0) return XCT_OK;
   const int grid = work < sms * per_sm ? work : sms * per_sm;
-  XCT_TRY_CUDA(cudaMemsetAsync(a.work, 0, sizeof(int), st));
+  if (!list[0].work_zeroed) XCT_TRY_CUDA(cudaMemsetAsync(a.work, 0, sizeof(int), st));
   spmm_pipe_kernel<TX, TW, ST, WIDE, PAIR><<<grid, C::NT, smem, st>>>(a);
   count_launch();
   XCT_TRY_CUDA(cudaGetLastError());
@@ -1018,7 +1018,177 @@ xct_status pipe_any(const SpmmArgs* list, int count, cudaStream_t s) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// Direct form for few blocks and 16-byte staged rows (4 FP32 or 8 16-bit
+// slices: also one or two, padded).
+//
+// With fewer blocks than the persistent kernel has CTAs resident, every CTA
+// takes one block and its stages' latencies add up (claim, descriptor,
+// copies: 26 us for 360 blocks of 128^2 x 180, whose matrix lies in L2).
+// Here a block's whole footprint is gathered into shared memory at once, and
+// each lane then reads the entries that the persistent kernel's lane would,
+// in its order, so every sum is the same bit for bit.
+// ---------------------------------------------------------------------------
+constexpr int kDirectThreads = kRowsPerBlock * 4;
+
+template <class TX, class TW>
+__global__ void __launch_bounds__(kDirectThreads)
+    spmm_direct_kernel(const int64_t* __restrict__ blk_stage, const int64_t* __restrict__ stage_pix,
+                       const int32_t* __restrict__ stage_np, const int32_t* __restrict__ pix,
+                       const uint4* __restrict__ seg, const void* __restrict__ entries, int cap, int64_t nrows,
+                       int64_t ncols, const unsigned char* __restrict__ xs, float* __restrict__ y,
+                       const uint32_t* __restrict__ in_max, int mat_scale_exp, double* __restrict__ dot) {
+  constexpr int ST = 16 / PBytes<TX>::v;       // slices of a row
+  constexpr bool W16 = PBytes<TW>::v == 2;
+  using E = typename std::conditional<W16, uint32_t, uint2>::type;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int b = blockIdx.x, tile = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rb = tid >> 2, el = tid & 3, quad = rb >> 2, gq = rb & 3;
+  const int64_t s0 = blk_stage[b], s1 = blk_stage[b + 1];
+  float acc[ST];
+#pragma unroll
+  for (int i = 0; i < ST; ++i) acc[i] = 0.0f;
+  if (s1 > s0) {
+    const int64_t p0 = stage_pix[s0];
+    const int n = (int)(s1 - 1 - s0) * cap + stage_np[s1 - 1];
+    const uint4* xt = reinterpret_cast<const uint4*>(xs + (size_t)tile * ncols * 16);
+    uint4* xb = reinterpret_cast<uint4*>(smem);
+    for (int i = tid; i < n; i += kDirectThreads) xb[i] = __ldg(xt + __ldg(pix + p0 + i));
+    uint4 sg = __ldg(seg + s0 * kQuads + quad);
+    __syncthreads();
+    for (int64_t s = s0; s < s1; ++s, xb += cap) {
+      const int64_t off = (int64_t)(((uint64_t)sg.y << 32) | sg.x);
+      const uint32_t cw = gq < 2 ? sg.z : sg.w;
+      const int nch = ((int)((cw >> ((gq & 1) * 16)) & 0xffffu) + 3) >> 2;
+      const E* ep = reinterpret_cast<const E*>(entries) + off + gq * 4 + el;
+      if (s + 1 < s1) sg = __ldg(seg + (s + 1) * kQuads + quad);
+      for (int c = 0; c < nch; c += 8) {
+        E ev[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c + u < nch) ev[u] = __ldg(ep + (c + u) * 16);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (c + u < nch) {
+            const int at = (int)(eoff(ev[u]) / (uint32_t)kEntryRowBytes);
+            // (a padding entry adds 0 times the zero row)
+            if (at < cap) PFma<TX, TW, ST>::run(acc, xb[at], eval(ev[u]));
+          }
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1)
+#pragma unroll
+    for (int i = 0; i < ST; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+  float r[ST];
+#pragma unroll
+  for (int i = 0; i < ST; ++i) {
+    float scale = 1.0f;
+    if constexpr (PBytes<TX>::v == 2)
+      scale = ldexpf(1.0f, ceil_log2_exp_p(__uint_as_float(__ldg(in_max + tile * ST + i))) - mat_scale_exp);
+    else if constexpr (W16)
+      scale = ldexpf(1.0f, -mat_scale_exp);
+    r[i] = acc[i] * scale;
+  }
+  const int64_t row = (int64_t)b * kRowsPerBlock + rb;
+  if (row < nrows && el == 0) {
+    float4* dst = reinterpret_cast<float4*>(y + ((size_t)tile * nrows + row) * ST);
+#pragma unroll
+    for (int q = 0; q < ST / 4; ++q) dst[q] = make_float4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+  }
+  if (dot) {
+    // per-slice squared norms as the persistent kernel forms them (FP64 for
+    // FP32 rows, FP32 pairs for 16-bit ones): the four lanes of a row hold
+    // the same sums, each squares ST / 4 slices
+    constexpr bool X16 = PBytes<TX>::v == 2;
+    constexpr int DN = ST / 4;
+    using D = typename std::conditional<X16, Ff, double>::type;
+    __shared__ D red[kDirectThreads / 32][ST];
+    D d[DN];
+#pragma unroll
+    for (int i = 0; i < ST; ++i)
+      if (i / DN == el) {
+        if constexpr (X16)
+          d[i % DN] = ff_square(acc[i]);
+        else
+          d[i % DN] = (double)r[i] * (double)r[i];
+      }
+    int base = 0;
+    halve_rows<DN, 4>(d, lane, base);
+    constexpr int NF = halved_count(DN, 4), DUP = halved_dup_mask(DN, 4);
+    if ((lane & DUP) == 0)
+#pragma unroll
+      for (int i = 0; i < NF; ++i) red[warp][el * DN + base + i] = d[i];
+    __syncthreads();
+    if (tid < ST) {
+      double t;
+      if constexpr (X16) {
+        Ff f = red[0][tid];
+        for (int w = 1; w < kDirectThreads / 32; ++w) f = sum2(f, red[w][tid]);
+        t = ldexp((double)f.h + (double)f.l,
+                  2 * (ceil_log2_exp_p(__uint_as_float(__ldg(in_max + tile * ST + tid))) - mat_scale_exp));
+      } else {
+        t = 0.0;
+        for (int w = 0; w < kDirectThreads / 32; ++w) t += red[w][tid];
+      }
+      dot[(size_t)(tile * ST + tid) * gridDim.x + b] = t;
+    }
+  }
+}
+
+constexpr size_t kDirectSmem = 100 * 1024;   // two CTAs of the largest footprint share an SM
+
+template <class TX, class TW>
+xct_status launch_direct(const SpmmArgs& a, cudaStream_t st) {
+  const Layout& L = *a.L;
+  const size_t smem = (size_t)(L.fp_max > 0 ? L.fp_max : 1) * 16;
+  int dev = 0;
+  XCT_TRY_CUDA(cudaGetDevice(&dev));
+  static std::atomic<bool> configured[kMaxDevices];
+  if (dev < 0 || dev >= kMaxDevices || !configured[dev].load()) {
+    XCT_TRY_CUDA(cudaFuncSetAttribute(spmm_direct_kernel<TX, TW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kDirectSmem));
+    if (dev >= 0 && dev < kMaxDevices) configured[dev].store(true);
+  }
+  const unsigned char* src = PBytes<TX>::v == 2 ? reinterpret_cast<const unsigned char*>(a.staged16)
+                                               : reinterpret_cast<const unsigned char*>(a.x);
+  spmm_direct_kernel<TX, TW><<<dim3(L.nblocks, a.ntiles), kDirectThreads, smem, st>>>(
+      L.blk_stage, L.stage_pix, L.stage_np, L.pix, reinterpret_cast<const uint4*>(L.seg), L.ent, L.cap, L.nrows,
+      L.ncols, src, a.y, a.in_max, a.mat_scale_exp, a.dot_partial);
+  count_launch();
+  XCT_TRY_CUDA(cudaGetLastError());
+  return XCT_OK;
+}
+
 }  // namespace
+
+// One wave of blocks, 16-byte rows, a footprint that fits.
+bool spmm_direct_applies(const SpmmArgs& a) {
+  const Layout& L = *a.L;
+  const int pixb = a.st * (stages16(a.storage) ? 2 : 4);
+  if (pixb != 16 || L.unit != kEntryRowBytes || L.pair || L.nblocks == 0 ||
+      (matrix16(a.storage) && !stages16(a.storage)))
+    return false;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return (int64_t)L.nblocks * a.ntiles <= (int64_t)sms * kPipeMinb16 && L.fp_max * 16 <= (int64_t)kDirectSmem;
+}
+
+xct_status spmm_direct(const SpmmArgs& a, cudaStream_t s) {
+  switch (a.storage) {
+    case XCT_F32: return launch_direct<float, float>(a, s);
+    case XCT_F16: return launch_direct<__half, __half>(a, s);
+    case XCT_BF16: return launch_direct<__nv_bfloat16, __nv_bfloat16>(a, s);
+    default:
+      set_error("direct product: 16-bit matrices with FP32 vectors have no 16-byte rows");
+      return XCT_ERR_UNSUPPORTED;
+  }
+}
 
 // The persistent form needs 16-byte lane vectors, staged rows of 16, 32, 64
 // or 128 bytes and two buffers in the shared memory of one of its CTAs.

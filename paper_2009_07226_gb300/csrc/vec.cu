@@ -2,6 +2,8 @@
 // slice-major natural order and the internal [tile][ordered row][slice]
 // layout, and the CGLS vector updates and FP64 scalars (Eq. 1 with R = 0,
 // CGLS form with one initial back projection, per-slice scalars).
+#include <algorithm>
+
 #include "ff.cuh"
 #include "xct_internal.cuh"
 #include "xct_vec.cuh"
@@ -71,25 +73,36 @@ __global__ void __launch_bounds__(kConvThreads) to_natural_kernel(
 // Per-block partial sums are reduced in a fixed order (deterministic).
 // ---------------------------------------------------------------------------
 
+// part[W], pmax[W] per thread -> per-slice block totals.  Threads `per` = st /
+// W apart hold the same slices: lanes by shuffles, then the warps in order
+// through shared memory (one thread adding 256 pairs per slice took most of
+// a small vector's update: 20 -> 4 us a kernel at 128^2 x 180, one slice).
 template <int W>
-__device__ void block_slice_sums(const FF* part, const uint32_t* pmax, int st, int tile,
+__device__ void block_slice_sums(FF* part, uint32_t* pmax, int st, int tile,
                                  double* out_part, uint32_t* out_max, int nbx) {
-  // part[W], pmax[W] per thread -> per-slice block totals
-  __shared__ FF sd[kVecThreads * 4];
-  __shared__ uint32_t sm[kVecThreads * 4];
-  for (int w = 0; w < W; ++w) {
-    sd[threadIdx.x * W + w] = part ? part[w] : FF{0.0f, 0.0f};
-    sm[threadIdx.x * W + w] = pmax ? pmax[w] : 0u;
-  }
+  __shared__ FF sd[kVecThreads / 32][64];
+  __shared__ uint32_t sm[kVecThreads / 32][64];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = st / W;
+  for (int o = 16; o >= per; o >>= 1)
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      if (part) part[w] = ff_add(part[w], ff_shfl_xor(part[w], o));
+      if (pmax) pmax[w] = max(pmax[w], __shfl_xor_sync(0xffffffffu, pmax[w], o));
+    }
+  if (lane < per)
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      sd[warp][lane * W + w] = part ? part[w] : FF{0.0f, 0.0f};
+      sm[warp][lane * W + w] = pmax ? pmax[w] : 0u;
+    }
   __syncthreads();
-  const int per = st / W;  // threads sharing a slice set repeat every `per`
   for (int sl = threadIdx.x; sl < st; sl += blockDim.x) {
-    const int t0 = sl / W, w = sl % W;
-    FF acc{0.0f, 0.0f};
-    uint32_t mx = 0;
-    for (int t = t0; t < (int)blockDim.x; t += per) {
-      acc = ff_add(acc, sd[t * W + w]);
-      mx = max(mx, sm[t * W + w]);
+    FF acc = sd[0][sl];
+    uint32_t mx = sm[0][sl];
+    for (int k = 1; k < kVecThreads / 32; ++k) {
+      acc = ff_add(acc, sd[k][sl]);
+      mx = max(mx, sm[k][sl]);
     }
     const int gs = tile * st + sl;
     if (out_part) out_part[(size_t)gs * nbx + blockIdx.x] = ff_to_double(acc);
@@ -415,37 +428,42 @@ xct_status to_natural(const float* in, float* nat, const int32_t* inv_order, int
   return XCT_OK;
 }
 
-#define XCT_VEC_LAUNCH(KERNEL, ...)                                                   \
+#define XCT_VEC_LAUNCH(KERNEL, BLOCKS, ...)                                           \
   do {                                                                                \
-    dim3 grid_(kVecBlocks, (unsigned)ntiles);                                         \
+    dim3 grid_((unsigned)(BLOCKS), (unsigned)ntiles);                                         \
     if (st % 4 == 0) KERNEL<4><<<grid_, kVecThreads, 0, s>>>(__VA_ARGS__);            \
     else KERNEL<1><<<grid_, kVecThreads, 0, s>>>(__VA_ARGS__);                        \
     count_launch();                                                                   \
     XCT_TRY_CUDA(cudaGetLastError());                                                 \
   } while (0)
 
+int vec_blocks(int64_t rows, int st) {
+  const int64_t per = (int64_t)kVecThreads * (st % 4 == 0 ? 4 : 1);
+  return (int)std::min<int64_t>(std::max<int64_t>((rows * st + per - 1) / per, 1), kVecBlocks);
+}
+
 xct_status cgls_update_xr(float* x, const float* p, int64_t npix, float* r, const float* q,
                           int64_t nray, int st, int ntiles, const CglsScalars& sc, double* rpart,
-                          cudaStream_t s) {
-  XCT_VEC_LAUNCH(update_xr_kernel, x, p, npix * st, r, q, nray * st, st, sc.alpha, sc.max_r, rpart);
+                          int nblk, cudaStream_t s) {
+  XCT_VEC_LAUNCH(update_xr_kernel, nblk, x, p, npix * st, r, q, nray * st, st, sc.alpha, sc.max_r, rpart);
   return XCT_OK;
 }
 
 xct_status cgls_update_p(float* p, const float* sv, int64_t npix, int st, int ntiles,
                          const CglsScalars& sc, cudaStream_t s) {
-  XCT_VEC_LAUNCH(update_p_kernel, p, sv, npix * st, st, sc.beta, sc.max_p);
+  XCT_VEC_LAUNCH(update_p_kernel, vec_blocks(npix, st), p, sv, npix * st, st, sc.beta, sc.max_p);
   return XCT_OK;
 }
 
 xct_status cgls_residual(float* r, const float* q, int64_t nray, int st, int ntiles,
-                         uint32_t* max_r, double* rpart, cudaStream_t s) {
-  XCT_VEC_LAUNCH(residual_kernel, r, q, nray * st, st, max_r, rpart);
+                         uint32_t* max_r, double* rpart, int nblk, cudaStream_t s) {
+  XCT_VEC_LAUNCH(residual_kernel, nblk, r, q, nray * st, st, max_r, rpart);
   return XCT_OK;
 }
 
 xct_status vec_sub_sumsq(const float* q, const float* y, float* r, int64_t rows, int st,
                          int ntiles, uint32_t* max_r, double* rpart, cudaStream_t s) {
-  XCT_VEC_LAUNCH(sub_kernel, q, y, r, rows * st, st, max_r, rpart);
+  XCT_VEC_LAUNCH(sub_kernel, kVecBlocks, q, y, r, rows * st, st, max_r, rpart);
   return XCT_OK;
 }
 
@@ -456,9 +474,9 @@ xct_status vec_loss(const double* rpart, const double* tv, int S, double* out, c
   return XCT_OK;
 }
 
-xct_status cgls_init_scalars(const double* gpart, int nbg, const double* rpart,
+xct_status cgls_init_scalars(const double* gpart, int nbg, const double* rpart, int nbr,
                              const CglsScalars& sc, double* log, int S_pad, cudaStream_t s) {
-  cgls_init_kernel<<<S_pad, kVecThreads, 0, s>>>(gpart, nbg, rpart, kVecBlocks, sc, log, S_pad);
+  cgls_init_kernel<<<S_pad, kVecThreads, 0, s>>>(gpart, nbg, rpart, nbr, sc, log, S_pad);
   count_launch();
   XCT_TRY_CUDA(cudaGetLastError());
   return XCT_OK;
@@ -472,18 +490,18 @@ xct_status cgls_alpha(const double* dpart, int nbd, const CglsScalars& sc, int S
   return XCT_OK;
 }
 
-xct_status cgls_beta(const double* gpart, int nbg, const double* rpart, const CglsScalars& sc,
-                     double* log_k, int S_pad, cudaStream_t s) {
-  cgls_beta_kernel<<<S_pad, kVecThreads, 0, s>>>(gpart, nbg, rpart, kVecBlocks, sc, log_k);
+xct_status cgls_beta(const double* gpart, int nbg, const double* rpart, int nbr,
+                     const CglsScalars& sc, double* log_k, int S_pad, cudaStream_t s) {
+  cgls_beta_kernel<<<S_pad, kVecThreads, 0, s>>>(gpart, nbg, rpart, nbr, sc, log_k);
   count_launch();
   XCT_TRY_CUDA(cudaGetLastError());
   return XCT_OK;
 }
 
 xct_status cgls_restore(const double* gamma_in, const int32_t* active_in, int S,
-                        const double* rpart, const CglsScalars& sc, double* log, int S_pad,
+                        const double* rpart, int nbr, const CglsScalars& sc, double* log, int S_pad,
                         cudaStream_t s) {
-  cgls_restore_kernel<<<S_pad, kVecThreads, 0, s>>>(gamma_in, active_in, S, rpart, kVecBlocks, sc,
+  cgls_restore_kernel<<<S_pad, kVecThreads, 0, s>>>(gamma_in, active_in, S, rpart, nbr, sc,
                                                      log);
   count_launch();
   XCT_TRY_CUDA(cudaGetLastError());

@@ -221,6 +221,7 @@ struct Layout {
   int64_t nstages = 0;
   int64_t nslots = 0;          // stored entries including padding
   int64_t footprint = 0;       // staged vectors over all stages
+  int64_t fp_max = 0;          // staged vectors of the block with most
   int64_t* blk_stage = nullptr;   // [nblocks + 1] stage ranges of the blocks
   int64_t* stage_pix = nullptr;   // [nstages + 1] offsets into pix
   int32_t* stage_np = nullptr;    // [nstages] staged rows of each stage
@@ -397,6 +398,7 @@ struct SpmmArgs {
                            // normalised 16-bit copy of x (unused for FP32)
   int* work;               // scratch: one work counter (persistent form)
   int* err;                // device flag set to 1 if a bounded wait ran out
+  bool work_zeroed = false;   // the work counter is zero already
 };
 // The layout a product runs on: the matrix's wide-stage layout, where the
 // plan built one, for 16-byte staged rows of 16-bit slices; its paired
@@ -422,6 +424,9 @@ xct_status spmm_run(const SpmmArgs& a, cudaStream_t s);
 // apply to this layout / tile width (the caller then uses the staged form)
 bool spmm_pipe_applies(const SpmmArgs& a);
 xct_status spmm_pipe(const SpmmArgs& a, cudaStream_t s);
+// the direct form for a product of few blocks and 16-byte rows (spmm_pipe.cu)
+bool spmm_direct_applies(const SpmmArgs& a);
+xct_status spmm_direct(const SpmmArgs& a, cudaStream_t s);
 // several products (same storage type, 128-byte rows) in one persistent
 // launch sharing one work counter (list[0].work) -- the batched solver
 constexpr int kMaxPipeProducts = 8;
