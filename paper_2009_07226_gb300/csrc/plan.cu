@@ -1922,7 +1922,9 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
       Arena mem(s, true);
       OctLayout& out = which == 0 ? p.oa : p.oat;
       bool fits = false;
-      const xct_status st = build_oct_layout(which == 0 ? ma : mt, p.storage, which == 0, out, mem, &fits, s);
+      const FootprintOrder order{which == 0, which == 0 ? p.ray_inv : p.pix_inv, which == 0 ? p.pix_inv : p.ray_inv,
+                                 cs_dev, g.n, g.n_det, T};
+      const xct_status st = build_oct_layout(which == 0 ? ma : mt, p.storage, order, out, mem, &fits, s);
       if (st == XCT_ERR_OOM || (st == XCT_OK && !fits)) {
         mem.release();
         out = OctLayout{};

@@ -19,7 +19,7 @@
 // What bounds it (512^2 x 768 x 512, binary16, whole kernel): with 64 slices
 // the shared-memory data path, about 86% busy: 16 wavefronts a chunk for the
 // gathers, 3 for values and positions and 3 of conflicts, plus the copies'
-// writes.  0.70 ms per projection, 0.66 per back projection, against 1.25 /
+// writes.  0.67 ms per projection, 0.61 per back projection, against 1.25 /
 // 1.24 ms of the FMA kernel on the paired layouts (spmm_pipe.cu); 32 slices
 // 0.41 / 0.46 against 0.77 / 0.76, 16 slices 0.35 / 0.34 against 0.49 / 0.50
 // and 8 slices 0.34 / 0.32 against 0.45 / 0.43 ms, there closer to the

@@ -339,9 +339,18 @@ struct CsrView {
   const double* val;
   int64_t nrows, ncols;
 };
+// How a block's footprint is ordered in an octet layout (see
+// oct_order_kernel): the matrix's rows are rays (A) or pixels (A^T), with
+// their and the columns' natural ids.
+struct FootprintOrder {
+  bool rays;
+  const int32_t *row_inv, *col_inv;   // ordered -> natural ids
+  const double* cs;                   // device [angles][2]
+  int n, nd, tile;
+};
 // the octet layout of a matrix (octet_layout.cu); *fits is false, and
 // nothing kept, when its stage buffers would not fit a product's CTA
-xct_status build_oct_layout(const CsrView& m, xct_dtype storage, bool angle_rows, OctLayout& L,
+xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const FootprintOrder& order, OctLayout& L,
                             Arena& keep, bool* fits, cudaStream_t s);
 
 // The octet layout that a product of the plan's matrix (or its transpose)

@@ -98,3 +98,24 @@ def test_octet_product_unaligned_buffers(xct):
         xct.xct_project(p.handle, xs, ys, S)
         torch.cuda.synchronize()
     assert torch.equal(ys, want)
+
+
+def test_octet_product_of_wide_footprints(xct):
+    """Rays 8 pixels apart: a block of 128 rays crosses more groups of columns
+    than are ordered along them (8192), and the back projection's blocks
+    fewer."""
+    import scipy.sparse as sp
+    n, m, nd, S = 720, 16, 90, 9
+    rng = np.random.default_rng(5)
+    with xct.Plan(n, m, nd, "f16", cos_sin=inputs.angle_table(m), det_spacing=8.0) as p:
+        mats = [sp.csr_matrix((v, c, r), shape=s) for (r, c, v), s in
+                ((xct.xct_plan_export(p.handle, xct.XCT_EXPORT_A_STORED), (m * nd, n * n)),
+                 (xct.xct_plan_export(p.handle, xct.XCT_EXPORT_AT_STORED), (n * n, m * nd)))]
+        x, y = _vectors(rng, S, n * n, "f16"), _vectors(rng, S, m * nd, "f16")
+        got = [p.project(x.reshape(S, n, n).cuda()), p.backproject(y.reshape(S, m, nd).cuda())]
+    # the groups (4 x 2 pixels) of one Hilbert tile of rays, half a block
+    c = np.concatenate([mats[0][k * nd + 40:k * nd + 48].indices for k in range(8)])
+    assert len(np.unique(c // n // 2 * (n // 4) + c % n // 4)) > 8192
+    for g, mat, v in zip(got, mats, (x, y)):
+        g, v = g.cpu().double().numpy().reshape(S, -1), v.double().numpy()
+        assert np.all(np.abs(g - (mat @ v.T).T) <= 1e-5 * (abs(mat) @ np.abs(v).T).T + 1e-30)
