@@ -235,9 +235,9 @@ xct_status xct_backproject_f64(xct_plan_t plan, const double* y, double* x, int3
 
 /* CGLS flags. */
 #define XCT_CGLS_X0 1u        /* start from the x passed in (else from 0) */
-#define XCT_CGLS_NO_GRAPH 2u  /* launch kernels directly, no CUDA graph */
-#define XCT_CGLS_TIMING 4u    /* time each phase with CUDA events (implies
-                                 NO_GRAPH); read back with xct_plan_stats */
+#define XCT_CGLS_NO_GRAPH 2u  /* accepted; solves always launch directly */
+#define XCT_CGLS_TIMING 4u    /* time each phase with CUDA events; read back
+                                 with xct_plan_stats */
 
 /*
  * xct_cgls -- least squares min ||y_s - A x_s|| for each slice s (Eq. 1 with
@@ -250,8 +250,7 @@ xct_status xct_backproject_f64(xct_plan_t plan, const double* y, double* x, int3
  * receiving (||r_k||, ||A^T r_k||) per iteration and slice.
  * A slice whose gamma or delta becomes exactly 0 stops silently (its x is
  * final).  Returns XCT_ERR_BREAKDOWN only if every slice stopped at k = 0;
- * x then holds x0 (or zeros).  The iteration runs as one CUDA graph unless
- * flags say otherwise.
+ * x then holds x0 (or zeros).
  */
 xct_status xct_cgls(xct_plan_t plan, const float* y, float* x, int32_t S,
                     int32_t iters, uint32_t flags, double* resid, void* stream);
@@ -346,8 +345,7 @@ typedef struct {
  * count solved together: jobs sharing a plan (geometry) are concatenated into
  * one batch of slices (Sec. II-B: slices share A; Sec. III-A2: batches fused
  * into minibatches); every product phase of all geometries with the same
- * kernel configuration is one persistent launch over their combined work; the
- * whole batch runs as one CUDA graph (unless XCT_CGLS_NO_GRAPH).  Flags:
+ * kernel configuration is one persistent launch over their combined work.  Flags:
  * XCT_CGLS_X0, XCT_CGLS_NO_GRAPH, XCT_BATCH_AUTOTUNE.  Each job's result is
  * bit-identical to xct_cgls on the concatenation of the slices of all jobs of
  * its plan (same slice-tile width).  A slice whose A^T r_0 is zero stays at
