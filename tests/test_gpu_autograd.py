@@ -173,3 +173,18 @@ def test_native_reconstruction_vs_oracle(xct, kind, tol):
     assert hr[-1] < 0.1 * hr[0]
     assert dl <= tol
     assert dx <= 10 * tol
+
+
+@pytest.mark.parametrize("length", [1, 255, 2048, 2049, 1024 * 2048 + 5])
+def test_datafit_vector_lengths(xct, length):
+    """Residual and cost of vectors shorter and longer than the kernel's grid,
+    from unaligned buffers: the residual exactly, the cost to FP64."""
+    gen = torch.Generator().manual_seed(length)
+    q, y = (torch.randn(3 * length + 1, generator=gen).cuda()[1:].view(3, length) for _ in range(2))
+    r = torch.full((3 * length + 1,), float("nan"), device="cuda")[1:].view(3, length)
+    val = np.zeros(1)
+    xct.xct_datafit(q, y, r, length, 3, val)
+    assert torch.equal(r, q - y)
+    # squares and sums in FP32 pairs (2^-46), blocks in FP64
+    want = 0.5 * float((q - y).double().square().sum())
+    assert abs(val[0] - want) <= 1e-12 * want
