@@ -36,6 +36,9 @@ __global__ void __launch_bounds__(kConvThreads) to_internal_kernel(
   const int t = blockIdx.y, live = min(ST, S - t * ST);
   const int nr = (int)min((int64_t)R, rows - h0);
   const int r = threadIdx.x % R;
+  allow_next();
+  wait_previous();
+  nat = after_wait(nat);
   const float* src = nat + (size_t)t * ST * rows + (r < nr ? inv[h0 + r] : 0);
   if (threadIdx.x < ST) smax[threadIdx.x] = 0u;
   __syncthreads();
@@ -75,13 +78,16 @@ __global__ void __launch_bounds__(kConvThreads) to_natural_kernel(
   const int64_t h0 = (int64_t)blockIdx.x * R;
   const int t = blockIdx.y, live = min(ST, S - t * ST);
   const int nr = (int)min((int64_t)R, rows - h0);
+  allow_next();
+  wait_previous();
+  in = after_wait(in);
   const float* src = in + ((size_t)t * rows + h0) * ST;
 #pragma unroll 4
   for (int i = threadIdx.x; i < nr * (ST / V); i += kConvThreads) {
     const int row = i / (ST / V), sl = i % (ST / V) * V;
     if (sl >= live) continue;
     if constexpr (V == 4) {
-      const float4 v = __ldg(reinterpret_cast<const float4*>(src) + i);
+      const float4 v = reinterpret_cast<const float4*>(src)[i];
       buf[sl][row] = v.x;
       buf[sl + 1][row] = v.y;
       buf[sl + 2][row] = v.z;
@@ -172,6 +178,13 @@ __global__ void __launch_bounds__(kVecThreads) update_xr_kernel(
     float* __restrict__ x, const float* __restrict__ p, int64_t npix_len,
     float* __restrict__ r, const float* __restrict__ q, int64_t nray_len, int st,
     const double* __restrict__ alpha, uint32_t* __restrict__ max_r, double* __restrict__ rpart) {
+  allow_next();
+  wait_previous();
+  x = after_wait(x);
+  p = after_wait(p);
+  r = after_wait(r);
+  q = after_wait(q);
+  alpha = after_wait(alpha);
   const int tile = blockIdx.y;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * W;
   const int64_t start = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * W;
@@ -215,6 +228,11 @@ template <int W>
 __global__ void __launch_bounds__(kVecThreads) update_p_kernel(
     float* __restrict__ p, const float* __restrict__ s, int64_t npix_len, int st,
     const double* __restrict__ beta, uint32_t* __restrict__ max_p) {
+  allow_next();
+  wait_previous();
+  p = after_wait(p);
+  s = after_wait(s);
+  beta = after_wait(beta);
   const int tile = blockIdx.y;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * W;
   const int64_t start = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * W;
@@ -244,6 +262,10 @@ template <int W>
 __global__ void __launch_bounds__(kVecThreads) residual_kernel(
     float* __restrict__ r, const float* __restrict__ q, int64_t nray_len, int st,
     uint32_t* __restrict__ max_r, double* __restrict__ rpart) {
+  allow_next();
+  wait_previous();
+  r = after_wait(r);
+  q = after_wait(q);
   const int tile = blockIdx.y;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * W;
   const int64_t start = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * W;
@@ -280,6 +302,10 @@ __global__ void __launch_bounds__(kVecThreads) sub_kernel(const float* __restric
                                                           float* __restrict__ r, int64_t len, int st,
                                                           uint32_t* __restrict__ max_r,
                                                           double* __restrict__ rpart) {
+  allow_next();
+  wait_previous();
+  q = after_wait(q);
+  y = after_wait(y);
   const int tile = blockIdx.y;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x * W;
   const int64_t start = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * W;
@@ -393,6 +419,8 @@ __device__ double block_reduce_fixed(const double* part, int n) {
 __global__ void __launch_bounds__(kVecThreads) cgls_init_kernel(
     const double* gpart, int nbg, const double* rpart, int nbr, CglsScalars sc, double* log,
     int S_pad) {
+  allow_next();
+  wait_previous();
   const int gs = blockIdx.x;
   const double g = block_reduce_fixed(gpart + (size_t)gs * nbg, nbg);
   const double rr = block_reduce_fixed(rpart + (size_t)gs * nbr, nbr);
@@ -413,6 +441,8 @@ __global__ void __launch_bounds__(kVecThreads) cgls_init_kernel(
 // delta = ||q||^2; alpha = gamma / delta (0 for a stopped slice)
 __global__ void __launch_bounds__(kVecThreads) cgls_alpha_kernel(const double* dpart, int nbd,
                                                                  CglsScalars sc) {
+  allow_next();
+  wait_previous();
   const int gs = blockIdx.x;
   const double d = block_reduce_fixed(dpart + (size_t)gs * nbd, nbd);
   if (threadIdx.x == 0) {
@@ -427,6 +457,8 @@ __global__ void __launch_bounds__(kVecThreads) cgls_alpha_kernel(const double* d
 __global__ void __launch_bounds__(kVecThreads) cgls_beta_kernel(const double* gpart, int nbg,
                                                                 const double* rpart, int nbr,
                                                                 CglsScalars sc, double* log_k) {
+  allow_next();
+  wait_previous();
   const int gs = blockIdx.x;
   const double g = block_reduce_fixed(gpart + (size_t)gs * nbg, nbg);
   const double rr = block_reduce_fixed(rpart + (size_t)gs * nbr, nbr);
@@ -478,17 +510,16 @@ __global__ void cgls_save_kernel(const CglsScalars sc, int S, CglsStateHeader hd
 template <class F>
 xct_status by_width(int st, F f) {
   switch (st) {
-    case 1: f(std::integral_constant<int, 1>()); break;
-    case 2: f(std::integral_constant<int, 2>()); break;
-    case 4: f(std::integral_constant<int, 4>()); break;
-    case 8: f(std::integral_constant<int, 8>()); break;
-    case 16: f(std::integral_constant<int, 16>()); break;
-    case 32: f(std::integral_constant<int, 32>()); break;
-    case 64: f(std::integral_constant<int, 64>()); break;
+    case 1: XCT_TRY_CUDA(f(std::integral_constant<int, 1>())); break;
+    case 2: XCT_TRY_CUDA(f(std::integral_constant<int, 2>())); break;
+    case 4: XCT_TRY_CUDA(f(std::integral_constant<int, 4>())); break;
+    case 8: XCT_TRY_CUDA(f(std::integral_constant<int, 8>())); break;
+    case 16: XCT_TRY_CUDA(f(std::integral_constant<int, 16>())); break;
+    case 32: XCT_TRY_CUDA(f(std::integral_constant<int, 32>())); break;
+    case 64: XCT_TRY_CUDA(f(std::integral_constant<int, 64>())); break;
     default: return XCT_ERR_UNSUPPORTED;
   }
   count_launch();
-  XCT_TRY_CUDA(cudaGetLastError());
   return XCT_OK;
 }
 
@@ -498,8 +529,8 @@ xct_status to_internal(const float* nat, float* in, const int32_t* inv_order, in
                        int st, int ntiles, uint32_t* max_bits, cudaStream_t s) {
   return by_width(st, [&](auto w) {
     constexpr int ST = decltype(w)::value, R = conv_rows(ST);
-    to_internal_kernel<ST><<<dim3((unsigned)((rows + R - 1) / R), (unsigned)ntiles), kConvThreads, 0, s>>>(
-        nat, in, inv_order, rows, S, max_bits);
+    return launch_early(to_internal_kernel<ST>, dim3((unsigned)((rows + R - 1) / R), (unsigned)ntiles), kConvThreads, 0, s,
+                        nat, in, inv_order, rows, S, max_bits);
   });
 }
 
@@ -507,18 +538,17 @@ xct_status to_natural(const float* in, float* nat, const int32_t* inv_order, int
                       int st, int ntiles, cudaStream_t s) {
   return by_width(st, [&](auto w) {
     constexpr int ST = decltype(w)::value, R = conv_rows(ST);
-    to_natural_kernel<ST><<<dim3((unsigned)((rows + R - 1) / R), (unsigned)ntiles), kConvThreads, 0, s>>>(
-        in, nat, inv_order, rows, S);
+    return launch_early(to_natural_kernel<ST>, dim3((unsigned)((rows + R - 1) / R), (unsigned)ntiles), kConvThreads, 0, s,
+                        in, nat, inv_order, rows, S);
   });
 }
 
 #define XCT_VEC_LAUNCH(KERNEL, BLOCKS, ...)                                           \
   do {                                                                                \
     dim3 grid_((unsigned)(BLOCKS), (unsigned)ntiles);                                         \
-    if (st % 4 == 0) KERNEL<4><<<grid_, kVecThreads, 0, s>>>(__VA_ARGS__);            \
-    else KERNEL<1><<<grid_, kVecThreads, 0, s>>>(__VA_ARGS__);                        \
+    if (st % 4 == 0) XCT_TRY_CUDA(launch_early(KERNEL<4>, grid_, kVecThreads, 0, s, __VA_ARGS__)); \
+    else XCT_TRY_CUDA(launch_early(KERNEL<1>, grid_, kVecThreads, 0, s, __VA_ARGS__)); \
     count_launch();                                                                   \
-    XCT_TRY_CUDA(cudaGetLastError());                                                 \
   } while (0)
 
 int vec_blocks(int64_t rows, int st) {
@@ -569,25 +599,22 @@ xct_status vec_loss(const double* rpart, const double* tv, int S, double* out, c
 
 xct_status cgls_init_scalars(const double* gpart, int nbg, const double* rpart, int nbr,
                              const CglsScalars& sc, double* log, int S_pad, cudaStream_t s) {
-  cgls_init_kernel<<<S_pad, kVecThreads, 0, s>>>(gpart, nbg, rpart, nbr, sc, log, S_pad);
+  XCT_TRY_CUDA(launch_early(cgls_init_kernel, S_pad, kVecThreads, 0, s, gpart, nbg, rpart, nbr, sc, log, S_pad));
   count_launch();
-  XCT_TRY_CUDA(cudaGetLastError());
   return XCT_OK;
 }
 
 xct_status cgls_alpha(const double* dpart, int nbd, const CglsScalars& sc, int S_pad,
                       cudaStream_t s) {
-  cgls_alpha_kernel<<<S_pad, kVecThreads, 0, s>>>(dpart, nbd, sc);
+  XCT_TRY_CUDA(launch_early(cgls_alpha_kernel, S_pad, kVecThreads, 0, s, dpart, nbd, sc));
   count_launch();
-  XCT_TRY_CUDA(cudaGetLastError());
   return XCT_OK;
 }
 
 xct_status cgls_beta(const double* gpart, int nbg, const double* rpart, int nbr,
                      const CglsScalars& sc, double* log_k, int S_pad, cudaStream_t s) {
-  cgls_beta_kernel<<<S_pad, kVecThreads, 0, s>>>(gpart, nbg, rpart, nbr, sc, log_k);
+  XCT_TRY_CUDA(launch_early(cgls_beta_kernel, S_pad, kVecThreads, 0, s, gpart, nbg, rpart, nbr, sc, log_k));
   count_launch();
-  XCT_TRY_CUDA(cudaGetLastError());
   return XCT_OK;
 }
 

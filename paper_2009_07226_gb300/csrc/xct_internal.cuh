@@ -27,6 +27,37 @@ constexpr int kMaxDevices = 64;   // per-device caches of launch attributes
 extern std::atomic<int64_t> g_launches;
 inline void count_launch(int64_t k = 1) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
+// Launches that overlap their predecessor's tail.  A kernel launched with
+// launch_early may start once every block of the kernel before it on the
+// stream has called allow_next (or ended); it calls wait_previous before it
+// touches memory that other kernels write, and only constants of the plan
+// before that.  The predecessor's results are visible after the wait, and a
+// kernel that allows its successor waits itself, so order along the stream is
+// kept.  (Solves of one 128^2 slice are a chain of 40 kernels of 2 to 15 us.)
+__device__ __forceinline__ void allow_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// the pointer as a new value, made after the wait: loads through a __restrict__
+// parameter might otherwise be moved ahead of it
+template <class T>
+__device__ __forceinline__ T* after_wait(T* p) {
+  asm volatile("" : "+l"(p) : : "memory");
+  return p;
+}
+template <class... P, class... A>
+cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Device allocation through the configured allocator (by default
 // stream-ordered: working memory from the library's pool, memory that a plan
 // keeps from the device's default pool).  Returns nullptr and sets the error
