@@ -4,7 +4,8 @@
 // Built from the CSR of the plan in four passes over its column ids, one CTA
 // per block of kOctRows rows:
 //   1. the block's footprint (8-column groups) counted in a shared bitmap;
-//   2. the footprint listed and ordered, and every entry's position in it;
+//   2. the footprint listed, ordered and cut into stages, and every entry's
+//      position in it (stage * capacity + place in the stage);
 //   3. per stage and octet, the distinct columns counted (a warp per octet,
 //      its bitmaps in shared memory), hence the chunks;
 //   4. the chunks filled: every entry finds its column's rank among the
@@ -163,30 +164,117 @@ __global__ void __launch_bounds__(kThreads) oct_fp_fill_kernel(CsrView m, const 
   }
 }
 
+// The row of octet place p (0 .. 7 of octet o) of block b, or -1 past the matrix.
+__device__ __forceinline__ int64_t octet_row(int b, int o, int r, int angle_rows, int64_t nrows) {
+  const int64_t row = (int64_t)b * kOctRows + (o >> 3) * 64 + oct_row((o & 7) * 8 + r, angle_rows);
+  return row < nrows ? row : -1;
+}
+
 // Orders a block's groups so that a stage, a piece of the list, holds work for
 // all of the block's rows: for rays by the place of the group's tile along
 // the block's (middle) ray, for pixels by its angle tile.  In ascending ids a
 // stage is a square patch of the footprint, which some of the block's rays
 // miss: the busiest warp of a stage had twice the average's columns (512^2 x
-// 768: 1.5 to 1.9 times, and 1.1 to 1.2 in this order), and the largest stage
-// 1.9 times the average's chunks (1.5).  512^2 x 768, 64 slices: xct_project
-// 0.78 -> 0.73 ms, xct_backproject 0.73 -> 0.69; 1536^2 x 1024, 32 slices: 7.0
-// -> 6.6.  A tile's groups stay together, and so do most runs.  A group that reaches past the matrix's columns comes last,
-// where the descriptor expects it.
+// 768: 1.5 to 1.9 times, and 1.1 to 1.2 in this order).  512^2 x 768, 64
+// slices: xct_project 0.78 -> 0.73 ms, xct_backproject 0.73 -> 0.69; 1536^2 x
+// 1024, 32 slices: 7.0 -> 6.6.  A tile's groups stay together, and so do most
+// runs.  A group that reaches past the matrix's columns comes last, where the
+// descriptor expects it.
+//
+// A stage ends at `cap` rows, or before its chunks could pass kStageChunks (a
+// group's weight is its columns over the block's octets; an octet's last chunk
+// may be partly filled): near the rotation centre the same pixels meet many
+// rays, and stages of equal rows sized the buffers for 1.5 to 1.9 times the
+// average stage, at 384 rows at most.  With stages of up to 512 rows cut this
+// way, and chunks leaving L2 first (spmm_mma.cu): 512^2 x 768, 64 slices 0.73 ->
+// 0.69 and 0.69 -> 0.65 ms, 8 slices 0.35 -> 0.31; 1536^2 x 1024, 32 slices 6.6
+// -> 5.8 and 5.8 -> 4.2 ms.
 constexpr int kOrderMax = 8192;   // groups of a block that are ordered (else ids ascend)
-__global__ void __launch_bounds__(kThreads) oct_order_kernel(CsrView m, FootprintOrder o,
+constexpr int kStageColumns = (kStageChunks - kOcts) * 16;
+// Cuts a list of groups into stages: add(i, weight of the list's i-th group)
+// returns the group's place, stage * groups of a stage + place in the stage.
+struct StageCut {
+  int32_t* cut;   // first group of every stage
+  int gps;
+  int st = -1, in = 0;
+  uint32_t cols = 0;
+  __device__ uint32_t add(int i, uint32_t weight) {
+    if (st < 0 || in == gps || cols + weight > (uint32_t)kStageColumns) {
+      cut[++st] = i;
+      in = 0;
+      cols = 0;
+    }
+    cols += weight;
+    return (uint32_t)(st * gps + in++);
+  }
+};
+// shared memory for blocks of up to n groups (a power of two)
+constexpr size_t order_smem(int n) { return (size_t)n * (kOcts + 4); }
+__global__ void __launch_bounds__(kThreads) oct_order_kernel(CsrView m, FootprintOrder o, int cap, int nmax,
                                                              const int64_t* fp_off, int32_t* groups,
-                                                             int32_t* epos) {
-  extern __shared__ uint32_t key[];                                   // [a power of two]
-  const int64_t f0 = fp_off[blockIdx.x];
-  const int n = (int)(fp_off[blockIdx.x + 1] - f0);
-  if (n < 2 || n > kOrderMax) return;
-  int n2 = 2;
-  while (n2 < n) n2 *= 2;
-  uint16_t* to = reinterpret_cast<uint16_t*>(key + n2);               // group -> place
+                                                             int32_t* epos, int32_t* cut, int64_t* nst) {
+  extern __shared__ uint32_t sm[];
+  const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gps = cap / 8;
+  const int64_t f0 = fp_off[b];
+  const int64_t nf = fp_off[b + 1] - f0;
   int64_t e0, e1;
   block_entries(m, &e0, &e1);
-  const int64_t mid = min((int64_t)blockIdx.x * kOctRows + kOctRows / 2, m.nrows - 1);
+  if (nf > nmax && nf <= 5 * nmax) {
+    // ids ascend; a group's weight is its entries (at least its columns)
+    for (int i = threadIdx.x; i < nf; i += blockDim.x) sm[i] = 0u;
+    __syncthreads();
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) atomicAdd(&sm[epos[e] >> 3], 1u);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      StageCut c{cut + f0, gps};
+      for (int g = 0; g < (int)nf; ++g) sm[g] = c.add(g, sm[g]);
+      nst[b] = c.st + 1;
+    }
+    __syncthreads();
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
+      const int32_t p = epos[e];
+      epos[e] = (int32_t)(sm[p >> 3] * 8 + (p & 7));
+    }
+    return;
+  }
+  if (nf == 0 || nf > nmax) {
+    const int64_t ns = (nf + gps - 1) / gps;
+    for (int64_t k = threadIdx.x; k < ns; k += blockDim.x) cut[f0 + k] = (int32_t)(k * gps);
+    if (threadIdx.x == 0) nst[b] = ns;
+    return;
+  }
+  const int n = (int)nf;
+  uint32_t* weight = sm;              // [nmax]
+  uint32_t* bits = sm + nmax;         // [octet][nmax / 4]: 8 columns of a group
+  uint32_t* key = bits;               // [nmax], after the bits
+  uint32_t* place = bits + nmax;      // [nmax]
+  for (int i = threadIdx.x; i < nmax * (kOcts / 4 + 1); i += blockDim.x) sm[i] = 0u;
+  __syncthreads();
+  uint32_t* own = bits + warp * (nmax / 4);
+  for (int r = 0; r < 8; ++r) {
+    const int64_t row = octet_row(b, warp, r, o.rays, m.nrows);
+    if (row < 0) continue;
+    const int64_t r0 = m.rowptr[row], r1 = m.rowptr[row + 1];
+    for (int64_t e = r0 + lane; e < r1; e += 32) {
+      const int32_t p = epos[e];
+      if (e > r0 && epos[e - 1] == p) {
+        atomicAdd(&weight[p >> 3], 1u);   // a repeated entry has a column of its own
+      } else {
+        const uint32_t bit = 1u << (p & 31);
+        if (!(own[p >> 5] & bit)) atomicOr(&own[p >> 5], bit);
+      }
+    }
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    uint32_t c = 0;
+    for (int w = 0; w < kOcts; ++w) c += __popc(bits[w * (nmax / 4) + (i >> 2)] >> (8 * (i & 3)) & 0xffu);
+    weight[i] += c;
+  }
+  __syncthreads();
+  int n2 = 2;
+  while (n2 < n) n2 *= 2;
+  const int64_t mid = min((int64_t)b * kOctRows + kOctRows / 2, m.nrows - 1);
   const int k_mid = o.rays ? o.row_inv[mid] / o.nd : 0;
   const float dx = o.rays ? -(float)o.cs[2 * k_mid + 1] : 0.0f, dy = o.rays ? (float)o.cs[2 * k_mid] : 0.0f;
   for (int i = threadIdx.x; i < n2; i += blockDim.x) {
@@ -195,14 +283,14 @@ __global__ void __launch_bounds__(kThreads) oct_order_kernel(CsrView m, Footprin
       const int64_t g = groups[f0 + i];
       if ((g + 1) * 8 <= m.ncols) {
         const int32_t id = o.col_inv[g * 8];
-        int place;
+        int at;
         if (o.rays) {
           const int ix = id % o.n / o.tile * o.tile, iy = id / o.n / o.tile * o.tile;
-          place = (int)floorf((float)ix * dx + (float)iy * dy) + 2 * o.n;
+          at = (int)floorf((float)ix * dx + (float)iy * dy) + 2 * o.n;
         } else {
-          place = id / o.nd / o.tile;
+          at = id / o.nd / o.tile;
         }
-        k = (uint32_t)min(max(place, 0), (1 << 19) - 2) << 13 | (uint32_t)i;
+        k = (uint32_t)min(max(at, 0), (1 << 19) - 2) << 13 | (uint32_t)i;
       } else {
         k = 0xffffe000u | (uint32_t)i;
       }
@@ -214,16 +302,23 @@ __global__ void __launch_bounds__(kThreads) oct_order_kernel(CsrView m, Footprin
   for (int span = 2; span <= n2; span *= 2)
     for (int d = span / 2; d > 0; d /= 2) {
       for (int i = threadIdx.x; i < n2 / 2; i += blockDim.x) {
-        const int a = (i / d) * 2 * d + i % d, b = a + d;
-        const uint32_t u = key[a], v = key[b];
-        if ((u > v) == ((a & span) == 0)) {
-          key[a] = v;
-          key[b] = u;
+        const int lo = (i / d) * 2 * d + i % d, hi = lo + d;
+        const uint32_t u = key[lo], v = key[hi];
+        if ((u > v) == ((lo & span) == 0)) {
+          key[lo] = v;
+          key[hi] = u;
         }
       }
       __syncthreads();
     }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) to[key[i] & (kOrderMax - 1)] = (uint16_t)i;
+  if (threadIdx.x == 0) {
+    StageCut c{cut + f0, gps};
+    for (int i = 0; i < n; ++i) {
+      const int g = key[i] & (kOrderMax - 1);
+      place[g] = c.add(i, weight[g]);
+    }
+    nst[b] = c.st + 1;
+  }
   // the list itself, in place: read, then written
   int32_t mine[kOrderMax / kThreads];
 #pragma unroll
@@ -239,14 +334,21 @@ __global__ void __launch_bounds__(kThreads) oct_order_kernel(CsrView m, Footprin
   }
   for (int64_t e = e0 + threadIdx.x; e < e1; e += kThreads) {
     const int32_t p = epos[e];
-    epos[e] = to[p >> 3] * 8 + (p & 7);
+    epos[e] = (int32_t)(place[p >> 3] * 8 + (p & 7));
   }
 }
 
-__global__ void oct_stage_count_kernel(const int64_t* fp_groups, int32_t nblocks, int32_t groups_per_stage,
-                                       int64_t* nst) {
-  const int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (b < nblocks) nst[b] = (fp_groups[b] + groups_per_stage - 1) / groups_per_stage;
+__global__ void oct_max_kernel(const int64_t* v, int32_t n, unsigned long long* out) {
+  const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) atomicMax(out, (unsigned long long)v[i]);
+}
+
+// the groups of stage k of the block whose groups are g[0 .. n), cut at cut[]
+__device__ __forceinline__ const int32_t* stage_groups(const int32_t* g, const int32_t* cut, int64_t k, int64_t ns,
+                                                       int64_t n, int* count) {
+  const int32_t at = cut[k];
+  *count = (int)((k + 1 < ns ? cut[k + 1] : n) - at);
+  return g + at;
 }
 
 // An octet's distinct columns in a stage as a bitmap over the stage's
@@ -276,12 +378,6 @@ struct OctCols {
 // place of the j-th column among an octet's g8 groups of 8 columns: columns
 // of one residue go to different groups
 __device__ __forceinline__ int oct_place(int j, int g8) { return (j % g8) * 8 + j / g8; }
-
-// The row of octet place p (0 .. 7 of octet o) of block b, or -1 past the matrix.
-__device__ __forceinline__ int64_t octet_row(int b, int o, int r, int angle_rows, int64_t nrows) {
-  const int64_t row = (int64_t)b * kOctRows + (o >> 3) * 64 + oct_row((o & 7) * 8 + r, angle_rows);
-  return row < nrows ? row : -1;
-}
 
 // Marks the octet's columns of stages [s0, s0 + kStageWindow) in the warp's
 // bitmaps and counts the repeated entries per stage.
@@ -349,12 +445,12 @@ __global__ void oct_stage_chunks_kernel(const int32_t* nch, int64_t nstages, int
 __device__ __forceinline__ bool run_starts(const int32_t* g, int i) { return i == 0 || g[i] != g[i - 1] + 1; }
 
 __global__ void oct_run_count_kernel(const int64_t* blk_stage, const int64_t* fp_off, const int64_t* fp_groups,
-                                     const int32_t* groups, int32_t nblocks, int gps, int* run_max) {
+                                     const int32_t* groups, const int32_t* cut, int* run_max) {
   const int b = blockIdx.x;
   for (int64_t s = blk_stage[b] + threadIdx.x; s < blk_stage[b + 1]; s += blockDim.x) {
-    const int64_t k = s - blk_stage[b];
-    const int32_t* g = groups + fp_off[b] + k * gps;
-    const int n = (int)min((int64_t)gps, fp_groups[b] - k * gps);
+    int n;
+    const int32_t* g = stage_groups(groups + fp_off[b], cut + fp_off[b], s - blk_stage[b],
+                                    blk_stage[b + 1] - blk_stage[b], fp_groups[b], &n);
     int r = 0;
     for (int i = 0; i < n; ++i) r += run_starts(g, i);
     atomicMax(run_max, r + 1);
@@ -362,14 +458,14 @@ __global__ void oct_run_count_kernel(const int64_t* blk_stage, const int64_t* fp
 }
 
 __global__ void oct_desc_kernel(const int64_t* blk_stage, const int64_t* fp_off, const int64_t* fp_groups,
-                                const int32_t* groups, const int32_t* nch, const int64_t* c0, int gps,
+                                const int32_t* groups, const int32_t* cut, const int32_t* nch, const int64_t* c0,
                                 int64_t ncols, int run_stride, int64_t desc_bytes, unsigned char* desc,
                                 uint2* chunks) {
   const int b = blockIdx.x;
   for (int64_t s = blk_stage[b] + threadIdx.x; s < blk_stage[b + 1]; s += blockDim.x) {
-    const int64_t k = s - blk_stage[b];
-    const int32_t* g = groups + fp_off[b] + k * gps;
-    const int n = (int)min((int64_t)gps, fp_groups[b] - k * gps);
+    int n;
+    const int32_t* g = stage_groups(groups + fp_off[b], cut + fp_off[b], s - blk_stage[b],
+                                    blk_stage[b + 1] - blk_stage[b], fp_groups[b], &n);
     OctStageHead h;
     h.c0 = c0[s];
     h.nch = (uint32_t)(c0[s + 1] - c0[s]);
@@ -498,7 +594,10 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
   XCT_TRY_CUDA(cudaStreamSynchronize(s));
   Arena tmp(s);
   int64_t *fp_groups, *fp_off, *nst;
-  int32_t *groups, *epos;
+  int32_t *groups, *epos, *cut;
+  unsigned long long *most, most_h = 0;   // groups of the block with most
+  XCT_TRY(tmp.get(&most, 1));
+  XCT_TRY_CUDA(cudaMemsetAsync(most, 0, sizeof(*most), s));
   XCT_TRY(tmp.get(&fp_groups, nb));
   XCT_TRY(tmp.get(&fp_off, nb + 1));
   XCT_TRY(tmp.get(&nst, nb));
@@ -508,25 +607,28 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
   oct_fp_count_kernel<<<nb, kThreads, count_smem, s>>>(m, fp_groups);
   count_launch();
   XCT_TRY(exclusive_scan_i64(fp_groups, fp_off, nb, s));
+  oct_max_kernel<<<grid_for(nb, 256), 256, 0, s>>>(fp_groups, nb, most);
+  count_launch();
+  XCT_TRY_CUDA(cudaMemcpyAsync(&most_h, most, sizeof(most_h), cudaMemcpyDeviceToHost, s));
   int64_t ngroups = 0;
   XCT_TRY_CUDA(cudaMemcpyAsync(&ngroups, fp_off + nb, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   XCT_TRY_CUDA(cudaStreamSynchronize(s));
   XCT_TRY(tmp.get(&groups, ngroups));
-  oct_fp_fill_kernel<<<nb, kThreads, fill_smem, s>>>(m, fp_off, groups, epos);
-  const int order_smem = kOrderMax * 6;
-  XCT_TRY_CUDA(cudaFuncSetAttribute(oct_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, order_smem));
-  oct_order_kernel<<<nb, kThreads, order_smem, s>>>(m, order, fp_off, groups, epos);
-  count_launch(2);
+  XCT_TRY(tmp.get(&cut, ngroups));
+  int nmax = 64;
+  while (nmax < (int64_t)most_h && nmax < kOrderMax) nmax *= 2;
+  XCT_TRY_CUDA(cudaFuncSetAttribute(oct_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)order_smem(nmax)));
   // stage capacity: the first at which two stage buffers of 128-byte rows
   // fit a CTA
-  for (int cap = kOctCap; cap >= 64; cap = cap * 3 / 4 / 64 * 64) {
+  for (int cap = kOctCap; cap >= 64; cap -= 64) {
     Arena own(s, true), part(s);
     L.cap = cap;
-    const int gps = cap / 8;
     const int bm_smem = kOcts * kStageWindow * cap / 8;
+    oct_fp_fill_kernel<<<nb, kThreads, fill_smem, s>>>(m, fp_off, groups, epos);
+    oct_order_kernel<<<nb, kThreads, order_smem(nmax), s>>>(m, order, cap, nmax, fp_off, groups, epos, cut, nst);
+    count_launch(2);
     XCT_TRY(own.get(&L.blk_stage, nb + 1));
-    oct_stage_count_kernel<<<grid_for(nb, 256), 256, 0, s>>>(fp_groups, nb, gps, nst);
-    count_launch();
     XCT_TRY(exclusive_scan_i64(nst, L.blk_stage, nb, s));
     XCT_TRY_CUDA(cudaMemcpyAsync(&L.nstages, L.blk_stage + nb, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     XCT_TRY_CUDA(cudaStreamSynchronize(s));
@@ -544,7 +646,7 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
     XCT_TRY_CUDA(cudaFuncSetAttribute(oct_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bm_smem));
     oct_count_kernel<<<nb, kThreads, bm_smem, s>>>(m, epos, L.blk_stage, cap, L.angle_rows, nch);
     oct_stage_chunks_kernel<<<grid_for(L.nstages, 256), 256, 0, s>>>(nch, L.nstages, total, emax);
-    oct_run_count_kernel<<<nb, 64, 0, s>>>(L.blk_stage, fp_off, fp_groups, groups, nb, gps, run_max);
+    oct_run_count_kernel<<<nb, 64, 0, s>>>(L.blk_stage, fp_off, fp_groups, groups, cut, run_max);
     count_launch(3);
     XCT_TRY(exclusive_scan_i32(total, c0, L.nstages, s));
     unsigned long long emax_h = 0;
@@ -560,7 +662,7 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
     XCT_TRY(own.get(&L.desc, (size_t)L.nstages * L.desc_bytes));
     XCT_TRY(own.get(&L.chunks, (size_t)L.nstages));
     XCT_TRY(own.get(&L.ent, (size_t)L.nchunks * kChunkBytes));
-    oct_desc_kernel<<<nb, 64, 0, s>>>(L.blk_stage, fp_off, fp_groups, groups, nch, c0, gps, m.ncols,
+    oct_desc_kernel<<<nb, 64, 0, s>>>(L.blk_stage, fp_off, fp_groups, groups, cut, nch, c0, m.ncols,
                                       run_stride, L.desc_bytes, L.desc, L.chunks);
     XCT_TRY_CUDA(cudaMemsetAsync(L.ent, 0, (size_t)L.nchunks * kChunkBytes, s));
     if (half_values(storage)) {

@@ -16,16 +16,17 @@
 // 16 consumer warps take one octet each and write its rows in the caller's
 // layout.
 //
-// What bounds it (512^2 x 768 x 512, binary16, whole kernel): with 64 slices
-// the shared-memory data path, about 86% busy: 16 wavefronts a chunk for the
-// gathers, 3 for values and positions and 3 of conflicts, plus the copies'
-// writes.  0.67 ms per projection, 0.61 per back projection, against 1.25 /
-// 1.24 ms of the FMA kernel on the paired layouts (spmm_pipe.cu); 32 slices
-// 0.41 / 0.46 against 0.77 / 0.76, 16 slices 0.35 / 0.34 against 0.49 / 0.50
-// and 8 slices 0.34 / 0.32 against 0.45 / 0.43 ms, there closer to the
-// chunks' stream from device memory (1.8 GB, 0.26 ms).  tcgen05 would want
-// 64 or more rows an operand tile, where only a tenth of the cells are
-// entries: more bytes from device memory than the sparse form needs.
+// What bounds it (512^2 x 768 x 512, binary16): with 64 slices the shared-memory
+// data path (16 wavefronts a chunk for the gathers, 3 for values and
+// positions and 3 of conflicts, plus the copies' writes): 0.69 ms per
+// xct_project, 0.65 per xct_backproject, 0.05 to 0.07 of them staging, against
+// 1.45 / 1.41 on the paired row layouts (spmm_pipe.cu) with their conversions;
+// 32 slices 0.41 / 0.38, 16 slices 0.33 / 0.32 and 8 slices 0.31 / 0.30 (the
+// FMA kernels alone 0.77 / 0.76, 0.49 / 0.50 and 0.45 / 0.43), there close to
+// the chunks' stream from device memory (1.8 GB, 0.26 ms).  At 1536^2 x 1024
+// the blocks' copies come from L2 at about 9 TB/s, its bound there.  tcgen05
+// would want 64 or more rows an operand tile, where only a tenth of the cells
+// are entries: more bytes from device memory than the sparse form needs.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -252,7 +253,10 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       if (lane == 0 && real) {
         mbar_expect_tx(&full[buf], xb + eb);
-        if (eb) bulk_g2s(ebuf(buf), src, eb, &full[buf]);
+        // chunks are read once, staged rows by many blocks: without the hint
+        // the chunks pushed them out of L2 (1536^2 x 1024: 16 slices 5.56 ->
+        // 5.10 ms, 32 slices 7.68 -> 7.11; 512^2 x 768, 64 slices: 1%)
+        if (eb) bulk_g2s_once(ebuf(buf), src, eb, &full[buf]);
       }
       __syncwarp();
       unsigned char* xd = xbuf(buf);

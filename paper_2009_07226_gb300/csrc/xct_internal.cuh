@@ -214,10 +214,12 @@ __host__ __device__ __forceinline__ int oct_row(int p, int angle_rows) {
   return (p & 48) | (p & 8) >> 1 | (p & 6) >> 1 | (p & 1) << 3;
 }
 constexpr int kChunkBytes = 256 + 32;
-// first stage capacity tried (projection of 64 slices at 512^2 x 768: 0.701
-// ms with 384, 0.708 with 256, 16 slices 0.352 and 0.443: the stage's fixed
-// costs; two buffers of 512 do not fit)
-constexpr int kOctCap = 384;
+// first stage capacity tried, and the chunks of a stage at which it ends early
+// (136: with 512 rows, two buffers of 128-byte rows, three of 64-byte ones and
+// four of 32-byte ones fit a CTA).  A stage's fixed costs want large stages:
+// projection of 8 slices at 512^2 x 768 0.35 ms with 384 rows, 0.46 with 256.
+constexpr int kStageChunks = 136;
+constexpr int kOctCap = 512;
 // A stage's descriptor: this head, the first chunk of every octet (kOcts + 1
 // numbers), padded to 16 bytes, then the runs of its staged rows as (first
 // column, first position) pairs and closing pairs (-1, positions).
