@@ -197,13 +197,14 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
     }
     // the end, once for every copy warp (only the first tells the consumers)
     for (int k = 0; k < NB && ok; ++k) ok = emit(k, kEnd, 0, 0, 0);
-    if (!ok) {
-      // let the descriptors already requested land before the CTA's shared
-      // memory goes away
-      if (lane == 0) atomicExch(a.err, 1);
-      for (uint32_t j = it > (uint32_t)kSlots ? it - kSlots : 0; j < it; ++j)
-        mbar_wait(&dbar[j % kSlots], (j / kSlots) & 1, kDrainNs);
-    }
+    // The descriptors requested land before the CTA's shared memory goes
+    // away, here too when every request was accepted: work that fits the
+    // slots is emitted without a wait, and a copy warp may have given up on
+    // its descriptor since.  (A slot's earlier requests were read before it
+    // was free for the last one.)
+    if (!ok && lane == 0) atomicExch(a.err, 1);
+    for (uint32_t j = it > (uint32_t)kSlots ? it - kSlots : 0; j < it; ++j)
+      mbar_wait(&dbar[j % kSlots], (j / kSlots) & 1, kDrainNs);
     return;
   }
   if (warp > kMmaWarps) {
@@ -223,7 +224,12 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
       const int ds = (int)(it % kSlots);
       bool ok = warp_wait(&dbar[ds], (it / kSlots) & 1, a.wait_ns);
       const int2 id = ident[ds];
-      if (ok && (id.y & kEnd) && id.x > 0) return;
+      if (ok && (id.y & kEnd) && id.x > 0) {
+        // the copies of this warp's last stage land first: consumers that
+        // gave up do not wait for them
+        if (use > 0) mbar_wait(&full[buf], (use - 1) & 1, kDrainNs);
+        return;
+      }
       const bool real = ok && (id.y & kReal) != 0;
       const unsigned char* dd = dslots + (size_t)ds * a.dbytes;
       const OctStageHead& dh = *reinterpret_cast<const OctStageHead*>(dd);
@@ -271,7 +277,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
         mbar_arrive(&full[buf]);   // the phase's single arrival; publishes the header
         mbar_arrive(&dfree[ds]);
       }
-      if (id.y & kEnd) return;
+      if (id.y & kEnd) return;   // (the stage before was consumed: the buffer was free)
     }
   }
 
