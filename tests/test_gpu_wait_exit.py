@@ -19,7 +19,7 @@ def xct():
 
 # a few stages in all (they fit the descriptor slots, so that no request is
 # waited for), and many
-@pytest.mark.parametrize("kind", ["f16"])
+@pytest.mark.parametrize("kind", ["f16", "f32"])   # octet and row products
 @pytest.mark.parametrize("n,m,nd", [(24, 24, 24), (96, 144, 100)])
 def test_products_right_after_one_that_gave_up(xct, kind, n, m, nd):
     S = 64
