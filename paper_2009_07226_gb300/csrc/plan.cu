@@ -507,14 +507,23 @@ __global__ void col_count_kernel(const int32_t* col, int64_t nnz, int32_t* ccoun
 __global__ void transpose_fill_kernel(const int64_t* rowptr, const int32_t* col, const double* val,
                                       int64_t nrow, unsigned long long* cursor, int32_t* trow,
                                       double* tval) {
-  // a warp per row
+  // A warp per row.  Entries of one pixel lie side by side in a row (a ray
+  // along a grid line may hold a pixel twice: it crosses that line once): the
+  // first of them takes the places of all, in the row's order, so that the
+  // places of a row's entries do not depend on which lane comes first.
   const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   if (r >= nrow) return;
-  const int64_t e1 = rowptr[r + 1];
-  for (int64_t e = rowptr[r] + (threadIdx.x & 31); e < e1; e += 32) {
-    unsigned long long p = atomicAdd(&cursor[col[e]], 1ull);
-    trow[p] = (int32_t)r;
-    tval[p] = val[e];
+  const int64_t e0 = rowptr[r], e1 = rowptr[r + 1];
+  for (int64_t e = e0 + (threadIdx.x & 31); e < e1; e += 32) {
+    const int32_t c = col[e];
+    if (e > e0 && col[e - 1] == c) continue;
+    int k = 1;
+    while (e + k < e1 && col[e + k] == c) ++k;
+    const unsigned long long p = atomicAdd(&cursor[c], (unsigned long long)k);
+    for (int i = 0; i < k; ++i) {
+      trow[p + i] = (int32_t)r;
+      tval[p + i] = val[e + i];
+    }
   }
 }
 
@@ -528,7 +537,8 @@ __global__ void max_count_kernel(const int32_t* c, int64_t n, int32_t* out) {
 }
 
 // Sort each column's entries by row (bitonic on (row << 32 | position) keys in
-// shared memory), making the transpose independent of atomic arrival order.
+// shared memory), making the transpose independent of atomic arrival order
+// (entries of one row keep their places, which follow the row's order).
 __global__ void __launch_bounds__(256) column_sort_kernel(const int64_t* colptr, int32_t* trow,
                                                           double* tval, int pow2) {
   extern __shared__ unsigned long long sk[];
@@ -1979,7 +1989,8 @@ struct Coo { int32_t r, c; double v; };
 
 xct_status to_canonical(std::vector<Coo>& coo, int64_t nrows, int64_t* rowptr, int32_t* col,
                         double* val, int64_t* nnz) {
-  std::sort(coo.begin(), coo.end(), [](const Coo& a, const Coo& b) {
+  // (repeated entries keep the order in which they are stored)
+  std::stable_sort(coo.begin(), coo.end(), [](const Coo& a, const Coo& b) {
     return a.r != b.r ? a.r < b.r : a.c < b.c;
   });
   *nnz = (int64_t)coo.size();
