@@ -603,7 +603,11 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
   XCT_TRY(tmp.get(&nst, nb));
   XCT_TRY(tmp.get(&epos, nnz));
   const int count_smem = kWinWords * 4, fill_smem = kWinWords * 8;
-  XCT_TRY_CUDA(cudaFuncSetAttribute(oct_fp_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, fill_smem));
+  XCT_TRY(allow_all_smem<oct_fp_fill_kernel>());
+  XCT_TRY(allow_all_smem<oct_order_kernel>());
+  XCT_TRY(allow_all_smem<oct_count_kernel>());
+  XCT_TRY(allow_all_smem<oct_fill_kernel<true>>());
+  XCT_TRY(allow_all_smem<oct_fill_kernel<false>>());
   oct_fp_count_kernel<<<nb, kThreads, count_smem, s>>>(m, fp_groups);
   count_launch();
   XCT_TRY(exclusive_scan_i64(fp_groups, fp_off, nb, s));
@@ -617,8 +621,6 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
   XCT_TRY(tmp.get(&cut, ngroups));
   int nmax = 64;
   while (nmax < (int64_t)most_h && nmax < kOrderMax) nmax *= 2;
-  XCT_TRY_CUDA(cudaFuncSetAttribute(oct_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)order_smem(nmax)));
   // stage capacity: the first at which two stage buffers of 128-byte rows
   // fit a CTA
   for (int cap = kOctCap; cap >= 64; cap -= 64) {
@@ -643,7 +645,6 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
     XCT_TRY(part.get(&run_max, 1));
     XCT_TRY_CUDA(cudaMemsetAsync(emax, 0, sizeof(unsigned long long), s));
     XCT_TRY_CUDA(cudaMemsetAsync(run_max, 0, sizeof(int), s));
-    XCT_TRY_CUDA(cudaFuncSetAttribute(oct_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bm_smem));
     oct_count_kernel<<<nb, kThreads, bm_smem, s>>>(m, epos, L.blk_stage, cap, L.angle_rows, nch);
     oct_stage_chunks_kernel<<<grid_for(L.nstages, 256), 256, 0, s>>>(nch, L.nstages, total, emax);
     oct_run_count_kernel<<<nb, 64, 0, s>>>(L.blk_stage, fp_off, fp_groups, groups, cut, run_max);
@@ -666,11 +667,9 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
                                       run_stride, L.desc_bytes, L.desc, L.chunks);
     XCT_TRY_CUDA(cudaMemsetAsync(L.ent, 0, (size_t)L.nchunks * kChunkBytes, s));
     if (half_values(storage)) {
-      XCT_TRY_CUDA(cudaFuncSetAttribute(oct_fill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bm_smem));
       oct_fill_kernel<true><<<nb, kThreads, bm_smem, s>>>(m, epos, L.blk_stage, cap, L.angle_rows, L.desc,
                                                           L.desc_bytes, L.ent);
     } else {
-      XCT_TRY_CUDA(cudaFuncSetAttribute(oct_fill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bm_smem));
       oct_fill_kernel<false><<<nb, kThreads, bm_smem, s>>>(m, epos, L.blk_stage, cap, L.angle_rows, L.desc,
                                                            L.desc_bytes, L.ent);
     }

@@ -613,9 +613,7 @@ xct_status transpose(const int64_t* rowptr, const int32_t* col, const double* va
       set_error("a column holds %d entries; the transpose sort handles at most 8192", hmax);
       return XCT_ERR_UNSUPPORTED;
     }
-    if (smem > 48 * 1024)
-      XCT_TRY_CUDA(cudaFuncSetAttribute(column_sort_kernel,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    XCT_TRY(allow_all_smem<column_sort_kernel>());
     if (hmax > 1) {
       column_sort_kernel<<<(unsigned)ncol, 256, smem, s>>>(colptr, trow, tval, p2);
       count_launch();

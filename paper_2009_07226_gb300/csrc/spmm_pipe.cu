@@ -945,17 +945,9 @@ xct_status launch_pipe(const SpmmArgs* list, int count, cudaStream_t st) {
     set_error("persistent product: %zu bytes of shared memory needed", smem);
     return XCT_ERR_UNSUPPORTED;
   }
-  // the opt-in shared-memory size is a per-device attribute: set it once per
-  // device and size
-  static std::atomic<int> configured_for[kMaxDevices];
-  int cur_dev = 0;
+  XCT_TRY((allow_all_smem<spmm_pipe_kernel<TX, TW, ST, WIDE, PAIR>>()));
+  int cur_dev = 0, sms = 0;
   XCT_TRY_CUDA(cudaGetDevice(&cur_dev));
-  if (cur_dev < 0 || cur_dev >= kMaxDevices || configured_for[cur_dev].load() != (int)smem + 1) {
-    XCT_TRY_CUDA(cudaFuncSetAttribute(spmm_pipe_kernel<TX, TW, ST, WIDE, PAIR>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (cur_dev >= 0 && cur_dev < kMaxDevices) configured_for[cur_dev].store((int)smem + 1);
-  }
-  int sms = 0;
   XCT_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, cur_dev));
   if (work == 0) return XCT_OK;
   const int grid = work < sms * per_sm ? work : sms * per_sm;

@@ -97,6 +97,27 @@ xct_status noalloc_reserve(int device);
     if (st_ != XCT_OK) return st_;     \
   } while (0)
 
+// Lets blocks of a kernel ask for all the dynamic shared memory that a block
+// may have, once per device.  (The limit belongs to the kernel, not to a
+// launch: set to the size of each launch, one host thread could lower it
+// between another's setting and launch.)
+template <auto* Kernel>
+xct_status allow_all_smem() {
+  static std::atomic<bool> done[kMaxDevices];
+  int dev = 0;
+  XCT_TRY_CUDA(cudaGetDevice(&dev));
+  const bool known = dev >= 0 && dev < kMaxDevices;
+  if (known && done[dev].load()) return XCT_OK;
+  cudaFuncAttributes at;
+  int most = 0;
+  XCT_TRY_CUDA(cudaFuncGetAttributes(&at, Kernel));
+  XCT_TRY_CUDA(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  XCT_TRY_CUDA(cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    most - (int)at.sharedSizeBytes));
+  if (known) done[dev].store(true);
+  return XCT_OK;
+}
+
 // A set of device allocations released together (in reverse order).
 struct Arena {
   struct Item { void* p; size_t n; };
