@@ -81,10 +81,13 @@ struct Trace {
 // that the array is resident there before the first call that relies on it.
 xct_status noalloc_reserve(int device);
 
+// (a failure is reported here: the runtime's record of it goes too, or the next
+// check of that record, here or in another library, would report it again)
 #define XCT_TRY_CUDA(call)                                                   \
   do {                                                                       \
     cudaError_t e_ = (call);                                                 \
     if (e_ != cudaSuccess) {                                                 \
+      cudaGetLastError();                                                    \
       ::xct::set_error("%s failed: %s (%s:%d)", #call, cudaGetErrorString(e_), \
                        __FILE__, __LINE__);                                  \
       return XCT_ERR_CUDA;                                                   \
