@@ -308,7 +308,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
 #pragma unroll
         for (int q = 0; q < HN; ++q) {
           const uint32_t mb = __ldg(im + 16 * i + 8 * q + g);
-          big |= mb >= 0x7f800000u;
+          // (or is so small, at most 2^-128, that its scale is infinite)
+          big |= mb >= 0x7f800000u || mb - 1u < 0x00200000u;
           scale[i * HN + q] = ldexpf(1.0f, ceil_log2_exp_p(__uint_as_float(mb)) - a.mat_scale_exp);
         }
       finite = !__any_sync(0xffffffffu, big != 0u);
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
             multiply(x, w[u]);
           }
       } else {
-        // a slice of this tile holds an infinity or NaN: 0 times it in a
+        // a slice of this tile is staged with infinities or NaN: 0 times it in a
         // chunk's unused cells would reach rows that do not cross it, so the
         // entries are taken one by one
         for (int c = c0; c < c0 + n; ++c)
