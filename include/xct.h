@@ -411,8 +411,13 @@ xct_status xct_plan_export(xct_plan_t plan, int32_t what, int64_t* rowptr,
 xct_status xct_plan_order(xct_plan_t plan, int32_t* pix, int32_t* ray);
 
 /*
- * Device memory.  By default the library allocates with cudaMallocAsync /
- * cudaFreeAsync on the call's stream.  A caller may route every allocation
+ * Device memory.  By default the library allocates on the call's stream in
+ * stream order: what a plan keeps from the device's default pool
+ * (cudaMallocAsync), the working memory of calls, while the device has plans,
+ * from a pool of the library's own, which holds up to 4 GiB of it mapped between
+ * calls.  That memory goes back to the device when the last plan is released
+ * and whenever an allocation of the library fails, which is then tried once
+ * more (not under stream capture).  A caller may route every allocation
  * through its own allocator (e.g. a framework's caching allocator); the
  * callbacks must be thread-safe and remain valid until reset.  alloc returns
  * NULL on failure (the library then returns XCT_ERR_OOM and frees what it

@@ -49,26 +49,34 @@ AllocHook hook() {
 }  // namespace
 
 // The working memory of a call comes from a pool of the library's own on each
-// device, which keeps up to kScratchKept bytes mapped across synchronisations:
-// CUDA's default pool unmaps everything free at each one, and mapping a
-// call's buffers again took 0.6 ms of a 2.0 ms call (512^2 x 768, 64 slices,
-// waited for) and a third of a small plan's build.  What it keeps goes back
-// to the device when the last plan is released.  Memory that plans keep comes
-// from the default pool, so that this one's size is that of the scratch alone.
+// device that has plans, which keeps up to kScratchKept bytes mapped across
+// synchronisations: CUDA's default pool unmaps everything free at each one,
+// and mapping a call's buffers again took 0.6 ms of a 2.0 ms call (512^2 x 768,
+// 64 slices, waited for) and a third of a small plan's build.  What it keeps
+// goes back to the device when an allocation fails and when the last plan is
+// released (or its build fails).  Memory that plans keep comes from the default
+// pool, so that this one's size is that of the scratch alone, and so does the
+// working memory of calls on a device without plans.
 namespace {
 constexpr uint64_t kScratchKept = 4ull << 30;
 std::mutex g_pool_mu;
 cudaMemPool_t g_pool[kMaxDevices] = {};
 int g_plans[kMaxDevices] = {};
 
-// the current device's pool; nullptr (the default pool serves) on any failure
-cudaMemPool_t scratch_pool() {
+int current_device() {
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
-    cudaGetLastError();
-    return nullptr;
-  }
+  if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) return dev;
+  cudaGetLastError();
+  return -1;
+}
+
+// the current device's pool; nullptr (the default pool serves) without plans
+// and on any failure
+cudaMemPool_t scratch_pool() {
+  const int dev = current_device();
+  if (dev < 0) return nullptr;
   std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (g_plans[dev] == 0) return nullptr;
   if (!g_pool[dev]) {
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
@@ -86,14 +94,28 @@ cudaMemPool_t scratch_pool() {
   }
   return g_pool[dev];
 }
+
+void trim_scratch(int dev) {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (g_pool[dev] && cudaMemPoolTrimTo(g_pool[dev], 0) != cudaSuccess) cudaGetLastError();
+}
+
+bool is_capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
 }  // namespace
 
 void scratch_plans(int device, int change) {
   if (device < 0 || device >= kMaxDevices) return;
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  g_plans[device] += change;
-  if (g_plans[device] == 0 && g_pool[device] && cudaMemPoolTrimTo(g_pool[device], 0) != cudaSuccess)
-    cudaGetLastError();
+  int left;
+  {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    left = g_plans[device] += change;
+  }
+  if (left == 0) trim_scratch(device);
 }
 
 void* dalloc(size_t bytes, cudaStream_t s, bool keep) {
@@ -104,10 +126,22 @@ void* dalloc(size_t bytes, cudaStream_t s, bool keep) {
     return p;
   }
   void* p = nullptr;
-  cudaMemPool_t pool = keep ? nullptr : scratch_pool();
-  cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, s) : cudaMallocAsync(&p, bytes, s);
+  auto attempt = [&]() {
+    cudaMemPool_t pool = keep ? nullptr : scratch_pool();
+    const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, s) : cudaMallocAsync(&p, bytes, s);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+  };
+  cudaError_t e = attempt();
+  const int dev = current_device();
+  if (e == cudaErrorMemoryAllocation && dev >= 0 && !is_capturing(s)) {
+    // once more with the scratch that lies free (what this stream's earlier
+    // calls released is free once they have run) back on the device
+    if (cudaStreamSynchronize(s) != cudaSuccess) cudaGetLastError();
+    trim_scratch(dev);
+    e = attempt();
+  }
   if (e != cudaSuccess) {
-    cudaGetLastError();
     set_error("cudaMallocAsync(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
     return nullptr;
   }
@@ -689,9 +723,14 @@ xct_status xct_plan(const xct_geometry* g, xct_dtype storage, uint32_t flags, vo
     set_error("no CUDA device");
     return XCT_ERR_CUDA;
   }
+  scratch_plans(p->device, 1);
   xct_status st = build_plan(*p, s);
   if (st != XCT_OK) {
     cudaStreamSynchronize(s);
+    const int device = p->device;
+    p.reset();
+    cudaStreamSynchronize(s);   // what the plan held is free, too
+    scratch_plans(device, -1);
     return st;
   }
   // the fixed array of xct_project_noalloc is loaded with its module on first
@@ -699,7 +738,6 @@ xct_status xct_plan(const xct_geometry* g, xct_dtype storage, uint32_t flags, vo
   // caller is still allowed to allocate (a failure here is reported again,
   // and only, by xct_project_noalloc)
   noalloc_reserve(p->device);
-  scratch_plans(p->device, 1);
   *out = p.release();
   return XCT_OK;
 }
