@@ -139,6 +139,15 @@ typedef struct xct_plan_s* xct_plan_t;
  * Traces every ray on the GPU (count pass, scan, fill pass), orders pixels
  * and rays along the pseudo-Hilbert curve, forms the explicit transpose
  * (stable in ray order), and packs both into the staged kernel layout.
+ * Plans of 16-bit slices (XCT_F16 / XCT_BF16) also hold octet layouts of A and
+ * A^T, dense pieces of 16 columns by 8 rows for the tensor cores, which
+ * xct_project, xct_backproject and xct_project_noalloc run on (the products of
+ * solves and xct_project_rows stay on the row layouts).  They take 1.2 to 1.6
+ * times the bytes of the row layouts (512^2 x 768 angles: 1.79 + 1.76 GB beside
+ * 1.42 + 1.35; 1536^2 x 1024: 32.0 + 21.5 beside 20.2 + 17.7).  Where device memory runs out while one is built, or its stages
+ * do not fit the product kernel, the plan does without it, and products of
+ * that matrix run on the row layouts: slower, and summed in another order
+ * (xct_stats tells which are there).
  * Synchronous: returns when the plan is ready (the work runs on `stream`).
  * `out` receives the plan; on error *out is NULL and nothing is leaked.
  */
@@ -365,7 +374,9 @@ typedef struct {
   int32_t stage_capacity_at;         /* rays of A^T per staged buffer */
   int64_t stages_a, stages_at;       /* staged buffers over all blocks */
   int64_t slots_a, slots_at;         /* stored entries incl. padding */
-  int64_t bytes_a, bytes_at;         /* device bytes of each packed form */
+  int64_t bytes_a, bytes_at;         /* device bytes of the row layouts (the
+                                        plan's own; not the wide-stage, paired
+                                        and octet layouts) */
   double plan_ms;                    /* wall time of xct_plan */
   /* filled by the last xct_cgls run with XCT_CGLS_TIMING: */
   double t_project_ms, t_backproject_ms, t_other_ms;
@@ -380,6 +391,9 @@ typedef struct {
      aside: the distinct columns of each pair of rows, summed over the stages
      (the plain layouts read one staged row per entry, nnz) */
   int64_t gathers_a_paired, gathers_at_paired;
+  /* device bytes of the octet layouts of A and A^T (XCT_F16 / XCT_BF16; see
+     xct_plan); 0: none, and products of that matrix run on its row layouts */
+  int64_t bytes_a_octets, bytes_at_octets;
 } xct_stats;
 
 xct_status xct_plan_stats(xct_plan_t plan, xct_stats* out);

@@ -1973,6 +1973,8 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   st.slots_at_paired = p.lat.paired ? p.lat.paired->nslots : 0;
   st.gathers_a_paired = p.la.paired ? p.la.paired->gathers : 0;
   st.gathers_at_paired = p.lat.paired ? p.lat.paired->gathers : 0;
+  st.bytes_a_octets = p.la.oct ? p.la.oct->bytes : 0;
+  st.bytes_at_octets = p.lat.oct ? p.lat.oct->bytes : 0;
   st.plan_ms = std::chrono::duration<double, std::milli>(t1 - t0).count();
   return XCT_OK;
 }

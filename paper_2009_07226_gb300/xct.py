@@ -59,7 +59,8 @@ class xct_stats(ctypes.Structure):
                 ("t_stage_ms", ctypes.c_double), ("t_vector_ms", ctypes.c_double),
                 ("t_scalar_ms", ctypes.c_double), ("slots_a_paired", ctypes.c_int64),
                 ("slots_at_paired", ctypes.c_int64), ("gathers_a_paired", ctypes.c_int64),
-                ("gathers_at_paired", ctypes.c_int64)]
+                ("gathers_at_paired", ctypes.c_int64), ("bytes_a_octets", ctypes.c_int64),
+                ("bytes_at_octets", ctypes.c_int64)]
 
 
 class xct_job(ctypes.Structure):
