@@ -86,7 +86,12 @@ typedef struct {
 
 typedef struct xct_plan_s* xct_plan_t;
 
-/* Plan flags. */
+/* Plan flags.  Those that choose among row layouts (XCT_PLAN_NARROW_TILES,
+ * XCT_PLAN_PAIRED_ROWS, the tile widths of XCT_PLAN_FEW_SLICES above 8) act on
+ * the products of solves, of the TV reconstruction and of xct_project_rows; a
+ * 16-bit plan's xct_project and xct_backproject run on its octet layouts, but
+ * for slice tiles of 8 of a plan with XCT_PLAN_FEW_SLICES and for plans with
+ * XCT_PLAN_ROWS_ONLY. */
 #define XCT_PLAN_KEEP_F64 1u  /* keep the FP64 CSR of A and A^T on the device
                                  for xct_plan_export (12 bytes per entry each) */
 #define XCT_PLAN_AUTOTUNE 2u  /* choose each matrix's stage capacity -- the
@@ -132,6 +137,12 @@ typedef struct xct_plan_s* xct_plan_t;
                                      kernel (they are then not kept).  Adds
                                      about 1.2x the packed entries of A and
                                      A^T to the plan (8 bytes a slot) */
+#define XCT_PLAN_ROWS_ONLY 32u  /* no octet layouts (see xct_plan): for plans
+                                   that only solve, whose products never read
+                                   them, or where memory is short.
+                                   xct_project and xct_backproject run on the
+                                   row layouts, every row summed in the order
+                                   of its stored entries */
 
 /*
  * xct_plan -- build the memoized operator (Sec. II-B memoization; Sec. III-A1

@@ -681,7 +681,7 @@ xct_status xct_plan(const xct_geometry* g, xct_dtype storage, uint32_t flags, vo
     return XCT_ERR_INVALID;
   }
   if (flags & ~(XCT_PLAN_KEEP_F64 | XCT_PLAN_AUTOTUNE | XCT_PLAN_FEW_SLICES | XCT_PLAN_NARROW_TILES |
-                XCT_PLAN_PAIRED_ROWS)) {
+                XCT_PLAN_PAIRED_ROWS | XCT_PLAN_ROWS_ONLY)) {
     set_error("unknown plan flags 0x%x", flags);
     return XCT_ERR_INVALID;
   }

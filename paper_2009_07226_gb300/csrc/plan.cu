@@ -1925,7 +1925,7 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   // octet layouts for products between natural vectors of 16-bit slices;
   // where device memory runs out or a stage does not fit, those products use
   // the layouts above
-  if (stages16(p.storage)) {
+  if (stages16(p.storage) && !(p.flags & XCT_PLAN_ROWS_ONLY)) {
     for (int which = 0; which < 2; ++which) {
       Arena mem(s, true);
       OctLayout& out = which == 0 ? p.oa : p.oat;

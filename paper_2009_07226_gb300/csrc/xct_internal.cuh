@@ -414,7 +414,7 @@ xct_status build_oct_layout(const CsrView& m, xct_dtype storage, const Footprint
 // between natural vectors runs on, for slice tiles of st; nullptr: it runs on
 // the row layouts (FP32 slices; 8-slice tiles of a plan with wide-stage
 // layouts, which stream fewer bytes: 0.20 - 0.23 ms against 0.31 at 512^2 x
-// 768; a matrix whose octet layout did not fit).  Products inside solves, and
+// 768; a matrix whose octet layout did not fit, or a plan that asked for none).  Products inside solves, and
 // those whose FP64 cost is reported, stay on the row layouts: they keep each
 // row's order of summation, so that logged residual norms and costs do not
 // move.
