@@ -108,6 +108,59 @@ bool is_capturing(cudaStream_t s) {
 }
 }  // namespace
 
+namespace {
+std::mutex g_oct_mu;                // guards the next and every plan's hold on its octets
+std::vector<Plan*> g_oct_plans;     // plans whose octet layouts may be given up
+thread_local int t_keep_octets = 0;
+
+// Gives up the octet layouts of the device's plans that nothing uses; false:
+// there are none.
+bool drop_octets(int dev) {
+  std::lock_guard<std::mutex> lk(g_oct_mu);
+  std::vector<Plan*> idle;
+  for (Plan* p : g_oct_plans)
+    if (p->device == dev && p->oct_users == 0 && !p->oct_pinned && (p->la.oct || p->lat.oct)) idle.push_back(p);
+  // products already enqueued on them, on whatever stream, end first
+  if (idle.empty() || cudaDeviceSynchronize() != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  for (Plan* p : idle) {
+    p->la.oct = p->lat.oct = nullptr;
+    p->oa = p->oat = OctLayout{};
+    p->stats.bytes_a_octets = p->stats.bytes_at_octets = 0;
+    p->oct_mem.stream = nullptr;
+    p->oct_mem.release();
+  }
+  if (cudaStreamSynchronize(nullptr) != cudaSuccess) cudaGetLastError();   // the memory is the device's again
+  return true;
+}
+}  // namespace
+
+OctUse::OctUse(Plan& p, bool transposed, int st, cudaStream_t s) : plan_(p), layout_(nullptr) {
+  std::lock_guard<std::mutex> lk(g_oct_mu);
+  if (st > 0) layout_ = octets_for(p, transposed, st);
+  if (!layout_) return;
+  ++p.oct_users;
+  if (!p.oct_pinned && is_capturing(s)) p.oct_pinned = true;
+}
+OctUse::~OctUse() {
+  if (!layout_) return;
+  std::lock_guard<std::mutex> lk(g_oct_mu);
+  --plan_.oct_users;
+}
+void octets_may_go(Plan& p) {
+  if (hook().alloc || !(p.la.oct || p.lat.oct)) return;   // a caller's allocator: its memory, its limits
+  std::lock_guard<std::mutex> lk(g_oct_mu);
+  g_oct_plans.push_back(&p);
+}
+void octets_stay(Plan& p) {
+  std::lock_guard<std::mutex> lk(g_oct_mu);
+  g_oct_plans.erase(std::remove(g_oct_plans.begin(), g_oct_plans.end(), &p), g_oct_plans.end());
+}
+KeepOctets::KeepOctets() { ++t_keep_octets; }
+KeepOctets::~KeepOctets() { --t_keep_octets; }
+
 void scratch_plans(int device, int change) {
   if (device < 0 || device >= kMaxDevices) return;
   int left;
@@ -140,6 +193,8 @@ void* dalloc(size_t bytes, cudaStream_t s, bool keep) {
     if (cudaStreamSynchronize(s) != cudaSuccess) cudaGetLastError();
     trim_scratch(dev);
     e = attempt();
+    // and without the octet layouts, which no call needs
+    if (e == cudaErrorMemoryAllocation && t_keep_octets == 0 && drop_octets(dev)) e = attempt();
   }
   if (e != cudaSuccess) {
     set_error("cudaMallocAsync(%zu bytes) failed: %s", bytes, cudaGetErrorString(e));
@@ -521,7 +576,7 @@ xct_status apply_pipelined(Plan& p, bool transposed, const float* in, float* out
   const int32_t* in_inv = transposed ? p.ray_inv : p.pix_inv;
   const int32_t* out_inv = transposed ? p.pix_inv : p.ray_inv;
   const int64_t nin = L.ncols, nout = L.nrows;
-  const OctLayout* oct = octets_for(p, transposed, st);
+  const OctUse oct(p, transposed, st, s);
   Arena ar(s);
   float *Xn[2] = {nullptr, nullptr}, *Yn[2] = {nullptr, nullptr}, *Xi[2], *Yi[2];
   uint32_t* mx[2];
@@ -606,7 +661,7 @@ xct_status apply_impl(Plan& p, bool transposed, const float* in, float* out, int
   const bool in_host = is_host_pointer(in), out_host = is_host_pointer(out);
   if ((in_host || out_host) && ntiles > 1 && !rows)
     return apply_pipelined(p, transposed, in, out, S, st, ntiles, in_host, out_host, s);
-  const OctLayout* oct = rows ? nullptr : octets_for(p, transposed, st);
+  const OctUse oct(p, transposed, rows ? 0 : st, s);   // (0: no tile width has one)
   Arena ar(s);
   DevView iv, ov;
   XCT_TRY(device_view(in, (size_t)S * nin, true, ar, s, iv));
@@ -738,14 +793,16 @@ xct_status xct_plan(const xct_geometry* g, xct_dtype storage, uint32_t flags, vo
   // caller is still allowed to allocate (a failure here is reported again,
   // and only, by xct_project_noalloc)
   noalloc_reserve(p->device);
+  octets_may_go(*p);
   *out = p.release();
   return XCT_OK;
 }
 
 void xct_free(xct_plan_t plan) {
   if (!plan) return;
+  octets_stay(*plan);
   cudaDeviceSynchronize();
-  plan->mem.stream = nullptr;
+  plan->mem.stream = plan->oct_mem.stream = nullptr;
   const int device = plan->device;
   delete plan;
   scratch_plans(device, -1);
@@ -1050,6 +1107,7 @@ xct_status xct_plan_stats(xct_plan_t plan, xct_stats* out) {
     set_error("out is NULL");
     return XCT_ERR_INVALID;
   }
+  std::lock_guard<std::mutex> lk(g_oct_mu);   // (giving octets up writes their bytes)
   *out = plan->stats;
   return XCT_OK;
 }

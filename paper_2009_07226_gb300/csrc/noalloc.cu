@@ -141,7 +141,7 @@ extern "C" xct_status xct_project_noalloc(xct_plan_t plan, const float* x, float
   uint32_t* mx = reinterpret_cast<uint32_t*>(b + b_xi + b_yi + b_h);
   int* work = reinterpret_cast<int*>(b + b_xi + b_yi + b_h + b_mx);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (const OctLayout* oct = octets_for(p, false, st))
+  if (const OctUse oct(p, false, st, s); oct)
     return oct_product(*oct, OctProduct{x, y, S, st, p.pix_inv, p.ray_inv, p.mat_scale_exp, mx, h16, work, p.err},
                        p.storage, s);
   // the maxima accumulate with atomicMax: they must start at zero every call

@@ -1926,6 +1926,8 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   // where device memory runs out or a stage does not fit, those products use
   // the layouts above
   if (stages16(p.storage) && !(p.flags & XCT_PLAN_ROWS_ONLY)) {
+    const KeepOctets others;
+    p.oct_mem.stream = s;
     for (int which = 0; which < 2; ++which) {
       Arena mem(s, true);
       OctLayout& out = which == 0 ? p.oa : p.oat;
@@ -1939,7 +1941,7 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
         continue;
       }
       XCT_TRY(st);
-      mem.move_to(keep);
+      mem.move_to(p.oct_mem);
       (which == 0 ? p.la : p.lat).oct = &out;
     }
   }

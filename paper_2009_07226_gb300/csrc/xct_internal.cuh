@@ -384,7 +384,10 @@ struct Plan {
   // kept FP64 matrices (ordered ids), only with XCT_PLAN_KEEP_F64
   int64_t* a_rowptr = nullptr; int32_t* a_col = nullptr; double* a_val = nullptr;
   int64_t* t_rowptr = nullptr; int32_t* t_col = nullptr; double* t_val = nullptr;
-  Arena mem{nullptr, true};      // everything above lives here
+  Arena mem{nullptr, true};      // everything above lives here, but for
+  Arena oct_mem{nullptr, true};  // the octet layouts (see OctUse)
+  int oct_users = 0;             // products being enqueued on them
+  bool oct_pinned = false;       // a captured graph refers to them
   xct_stats stats{};
   std::map<int, int> tile_choice;  // measured slice-tile width per slice count
 };
@@ -422,6 +425,32 @@ inline const OctLayout* octets_for(const Plan& p, bool transposed, int st) {
   const Layout& L = transposed ? p.lat : p.la;
   return stages16(p.storage) && !(st == 8 && L.wide) ? L.oct : nullptr;
 }
+
+// A product's hold on the octet layout that it runs on, while it is enqueued
+// (null: there is none).  When device memory runs out, the layouts of plans
+// that no product is being enqueued on, and that no captured graph refers to,
+// are given up (api.cu): solves and plans that would fit without them do.
+class OctUse {
+ public:
+  OctUse(Plan& p, bool transposed, int st, cudaStream_t s);
+  ~OctUse();
+  OctUse(const OctUse&) = delete;
+  OctUse& operator=(const OctUse&) = delete;
+  explicit operator bool() const { return layout_ != nullptr; }
+  const OctLayout& operator*() const { return *layout_; }
+
+ private:
+  Plan& plan_;
+  const OctLayout* layout_;
+};
+// a plan whose octet layouts may be given up; before it is released, no more
+void octets_may_go(Plan& p);
+void octets_stay(Plan& p);
+// in this thread, memory that runs out takes no other plan's octet layouts
+struct KeepOctets {
+  KeepOctets();
+  ~KeepOctets();
+};
 
 // plan building (plan.cu)
 xct_status build_plan(Plan& p, cudaStream_t s);

@@ -106,3 +106,112 @@ def test_plans_that_fell_back_from_octets(xct, kind):
         torch.cuda.synchronize()
         assert budget.live == {}
     assert {(True, False), (False, False)} <= seen
+
+
+# ---------------------------------------------------------------------------
+# memory that runs out after the plan was built
+# ---------------------------------------------------------------------------
+
+MB = 1 << 20
+
+
+def _free():
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _kept(xct, n, m):
+    """Bytes that a binary16 plan of n^2 x m angles keeps."""
+    b = _Budget()
+    xct.xct_set_allocator(b.alloc, b.release)
+    try:
+        with xct.Plan(n, m, n, "f16", cos_sin=inputs.angle_table(m)):
+            torch.cuda.synchronize()
+            return sum(b.live.values())
+    finally:
+        xct.xct_set_allocator(None, None)
+
+
+def _solve_at_the_limit(xct, p, S, idle, iters=2):
+    """CGLS of S slices with less memory free (beside the `idle` bytes of the
+    library's scratch pool) than its working memory needs, and enough with
+    the plan's octet layouts; returns (y, x, status)."""
+    n, m, nd = p.n, p.m, p.nd
+    g = torch.Generator(device="cuda").manual_seed(1)
+    y = torch.rand((S, m, nd), device="cuda", generator=g)
+    x = torch.empty((S, n, n), device="cuda")
+    st = p.stats()
+    octets = st["bytes_a_octets"] + st["bytes_at_octets"]
+    scratch = S * (12 * n * n + 8 * m * nd + 2 * (n * n + m * nd))
+    assert octets > 400 * MB and scratch > idle + octets
+    hold = torch.empty(_free() - (scratch - octets // 2 - idle), dtype=torch.uint8, device="cuda")
+    try:
+        xct.xct_cgls(p.handle, y, x, S, iters)
+        status = xct.XCT_OK
+    except xct.XctError as e:
+        status = e.status
+    del hold
+    torch.cuda.empty_cache()
+    return y, x, status
+
+
+def test_a_solve_takes_the_octets_memory(xct):
+    n, m, S = 256, 384, 2048
+    kept = _kept(xct, n, m)
+    img = torch.rand((20, n, n), device="cuda")
+    before = _free()
+    with xct.Plan(n, m, n, "f16", cos_sin=inputs.angle_table(m)) as p:
+        want = p.project(img)
+        y, x, status = _solve_at_the_limit(xct, p, S, before - _free() - kept)
+        assert status == xct.XCT_OK
+        assert p.stats()["bytes_a_octets"] == p.stats()["bytes_at_octets"] == 0
+        got = p.project(img)
+        assert float((got - want).norm() / want.norm()) <= 1e-6
+        with xct.Plan(n, m, n, "f16", cos_sin=inputs.angle_table(m), rows_only=True) as q:
+            assert torch.equal(x, q.cgls(y, 2))
+            assert torch.equal(got, q.project(img))
+            assert torch.equal(p.backproject(got), q.backproject(got))
+
+
+def test_captured_products_keep_their_octets(xct):
+    n, m, S = 256, 384, 2048
+    kept = _kept(xct, n, m)
+    img = torch.rand((20, n, n), device="cuda")
+    before = _free()
+    with xct.Plan(n, m, n, "f16", cos_sin=inputs.angle_table(m)) as p:
+        want = p.project(img)
+        idle = before - _free() - kept
+        out = torch.empty_like(want)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            p.project(img, out=out)
+        _, _, status = _solve_at_the_limit(xct, p, S, idle)
+        assert status == xct.XCT_ERR_OOM
+        assert p.stats()["bytes_a_octets"] > 0
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+        del graph
+
+
+def test_building_octets_takes_no_other_plans(xct):
+    """A second plan whose octets do not fit goes without; the first keeps
+    its own."""
+    n, m = 256, 384
+    cs = inputs.angle_table(m)
+    with xct.Plan(n, m, n, "f16", cos_sin=cs) as p:
+        st = p.stats()
+        # less and less room (the build's working memory lies idle in the
+        # scratch pool since the first build)
+        room = st["bytes_a"] + st["bytes_at"] + st["bytes_a_octets"]
+        for leave in range(room, 0, -32 * MB):
+            hold = torch.empty(_free() - leave, dtype=torch.uint8, device="cuda")
+            with xct.Plan(n, m, n, "f16", cos_sin=cs) as q:
+                sq = q.stats()
+            del hold
+            if sq["bytes_a_octets"] * sq["bytes_at_octets"] == 0:
+                break
+        assert sq["bytes_a_octets"] * sq["bytes_at_octets"] == 0
+        assert p.stats() == st
