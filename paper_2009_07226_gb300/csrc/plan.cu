@@ -340,25 +340,38 @@ __global__ void siddon_fill_kernel(GeomDev g, const int32_t* ray_inv, const int3
 // accumulates RN32(length) * x[s][pixel] in FP32.
 //
 // FP64 instructions would bound it (a trace step takes a dozen even so), so
-// the walk itself runs in 64-bit integers: crossing parameters in units of
-// 2^-bits with |alpha| < 2^60 units, each axis's crossings a constant step
-// apart, the first crossing and the step from FP64.  The parameters drift by
-// at most half a unit a crossing (n * 2^-bits / 2: 1e-13 at n = 512, 5e-10 at
-// the largest grid), far below a length's rounding to FP32.  Rays nearly
-// along an axis (a component below 1e-4, where a line on a grid line could
-// take either side) and directions that are not unit vectors are traced as
-// the plan builder traces them.
+// the walk itself runs in integers: crossing parameters in units of 2^-bits
+// with |alpha| < 2^60 units, each axis's crossings a constant step apart.  The
+// first crossing is the FP64 one; the step, 1 / |d|, is taken to 2^-32 of a
+// unit (its quotient in FP64 corrected by its remainder) and its fraction
+// added with carry, so n crossings add less than a unit (4e-15 at n = 2048,
+// 6e-14 at the largest grid), less than the rounding of the plan builder's
+// FP64 parameters.  (Steps of whole units drifted by half a unit a crossing,
+// 9e-10 on the largest grid.)  Rays nearly along an axis (a component below
+// 1e-4, where a line on a grid line could take either side) and directions
+// that are not unit vectors are traced as the plan builder traces them.
 // The slices are interleaved in tiles first, so a step reads one contiguous
 // piece of kMfSlices slices instead of as many distant words.
-// 256^2 x 384, 24 slices: 61.7 -> 0.83 ms a call (three tiles of 8; before,
-// every tile walked in FP64 and read each slice on its own).
+// 256^2 x 384, 24 slices: 61.7 -> 0.73 ms a call (three tiles of 8; before,
+// every tile walked in FP64 and read each slice on its own); steps of whole
+// units would take 0.72.
 constexpr int kMfSlices = 8;
 
 struct FxRay {
   long long cur, ax, ay, sx, sy, amax;   // start, next crossings, steps, end
+  uint32_t fx, fy;                       // the steps' fractions in 2^-32 units
   int ix, iy, nx, ny;                    // pixel, crossings left with the direction's sign
 };
 constexpr int kFxMiss = INT32_MIN, kFxExact = INT32_MIN + 1;   // FxRay::nx
+
+// a += s with their fractions u, f: three additions with carry
+__device__ __forceinline__ void fx_step(long long& a, uint32_t& u, long long s, uint32_t f) {
+  uint32_t lo = (uint32_t)a, hi = (uint32_t)((unsigned long long)a >> 32);
+  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
+      : "+r"(u), "+r"(lo), "+r"(hi)
+      : "r"(f), "r"((uint32_t)s), "r"((uint32_t)((unsigned long long)s >> 32)));
+  a = (long long)((unsigned long long)hi << 32 | lo);
+}
 
 __global__ void __launch_bounds__(128) fx_setup_kernel(GeomDev g, int64_t nray, int bits, FxRay* out) {
   const int64_t ray = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -378,8 +391,16 @@ __global__ void __launch_bounds__(128) fx_setup_kernel(GeomDev g, int64_t nray, 
     f.amax = fixed(r.amax);
     f.ax = wx.left ? fixed(plane_alpha(wx.i, r.half, r.px, r.dx)) : 0;
     f.ay = wy.left ? fixed(plane_alpha(wy.i, r.half, r.py, r.dy)) : 0;
-    f.sx = __double2ll_rn(fmin(fabs(yx) * unit, most));
-    f.sy = __double2ll_rn(fmin(fabs(yy) * unit, most));
+    // 1 / |d| in units: y is rounded, y (1 - d y) what it lacks (a step too
+    // long for the chord is cut: it is not taken)
+    auto step = [&](double d, double y, long long* whole, uint32_t* part) {
+      const double v = fmin(fabs(y) * unit, most), w = floor(v);
+      const double rest = (v - w) + fabs(y) * __fma_rn(-d, y, 1.0) * unit, c = floor(rest);
+      *whole = (long long)w + (long long)c;
+      *part = __double2uint_rd((rest - c) * 4294967296.0);
+    };
+    step(r.dx, yx, &f.sx, &f.fx);
+    step(r.dy, yy, &f.sy, &f.fy);
     // before its next crossing an axis is in the pixel on the near side of
     // the plane; without crossings, in the one of the chord's midpoint
     const double mid = 0.5 * (r.amin + r.amax);
@@ -460,6 +481,7 @@ __global__ void __launch_bounds__(128) matfree_project_kernel(GeomDev g, const F
     const int dx = f.nx > 0 ? 1 : -1, dy = f.ny > 0 ? n : -n;
     int nx = abs(f.nx), ny = abs(f.ny), pix = f.iy * n + f.ix;
     long long cur = f.cur, ax = nx ? f.ax : kNone, ay = ny ? f.ay : kNone;
+    uint32_t ux = 0x80000000u, uy = 0x80000000u;   // fractions of the next crossings
     // each segment's slices are loaded while the one before is added
     float lp = 0.0f;
     Piece<NS> tp{};
@@ -478,10 +500,12 @@ __global__ void __launch_bounds__(128) matfree_project_kernel(GeomDev g, const F
       cur = nxt;
       if (isx) {
         pix += dx;
-        ax = --nx > 0 ? ax + f.sx : kNone;
+        fx_step(ax, ux, f.sx, f.fx);
+        if (--nx <= 0) ax = kNone;
       } else {
         pix += dy;
-        ay = --ny > 0 ? ay + f.sy : kNone;
+        fx_step(ay, uy, f.sy, f.fy);
+        if (--ny <= 0) ay = kNone;
       }
     }
     if (lp > 0.0f) {

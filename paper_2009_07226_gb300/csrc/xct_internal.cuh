@@ -454,7 +454,7 @@ struct KeepOctets {
 
 // plan building (plan.cu)
 xct_status build_plan(Plan& p, cudaStream_t s);
-// y = A x without the stored matrix: every ray traced again (plan.cu)
+// y = A x without the stored matrix: every ray walked again (plan.cu)
 xct_status matfree_project(const Plan& p, const double* cs_dev, const float* x, float* y, int S,
                            cudaStream_t s);
 // x = A^T y without the stored matrix: pixel-driven, lengths from each
