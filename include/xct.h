@@ -211,8 +211,10 @@ xct_status xct_backproject(xct_plan_t plan, const float* y, float* x,
  * 16384 and 45 degrees, under the rounding to FP32 but for the shortest), and
  * a piece that close to min_seg may be kept by one and dropped by the other;
  * other rays have the stored lengths.  A comparison point and the form
- * for grids whose A does not fit in memory.  x, y: natural layouts, host or
- * device.  Synchronous.
+ * for grids whose A does not fit in memory: its working memory is bounded (72
+ * bytes a ray for at most 4 Mi rays, and a copy of at most 1 GiB of slices or
+ * of 8 slices), and where that is refused it goes without, more slowly.  x, y:
+ * natural layouts, host or device.  Synchronous.
  */
 xct_status xct_project_matfree(xct_plan_t plan, const float* x, float* y, int32_t S,
                                void* stream);

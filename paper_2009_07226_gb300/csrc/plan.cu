@@ -373,9 +373,10 @@ __device__ __forceinline__ void fx_step(long long& a, uint32_t& u, long long s, 
   a = (long long)((unsigned long long)hi << 32 | lo);
 }
 
-__global__ void __launch_bounds__(128) fx_setup_kernel(GeomDev g, int64_t nray, int bits, FxRay* out) {
-  const int64_t ray = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (ray >= nray) return;
+__global__ void __launch_bounds__(128) fx_setup_kernel(GeomDev g, int64_t ray0, int64_t count, int bits,
+                                                       FxRay* out) {
+  const int64_t at = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, ray = ray0 + at;
+  if (at >= count) return;
   FxRay f{};
   Ray r;
   if (!setup_row(g, (int32_t)ray, r)) {
@@ -413,7 +414,7 @@ __global__ void __launch_bounds__(128) fx_setup_kernel(GeomDev g, int64_t nray, 
     f.nx = r.dx > 0.0 ? wx.left : -wx.left;
     f.ny = r.dy > 0.0 ? wy.left : -wy.left;
   }
-  out[ray] = f;
+  out[at] = f;
 }
 
 // natural [S][npix] -> [tiles][npix][NS] (slices past S are zero)
@@ -466,12 +467,17 @@ struct ProjSink {
 template <int NS>
 __global__ void __launch_bounds__(128) matfree_project_kernel(GeomDev g, const FxRay* __restrict__ rays, int bits,
                                                               long long min_len, const float* __restrict__ xt,
-                                                              float* __restrict__ y, int S, int64_t nray) {
-  const int64_t ray = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (ray >= nray) return;
+                                                              float* __restrict__ y, int S, int64_t ray0,
+                                                              int64_t count, int64_t nray) {
+  const int64_t at = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, ray = ray0 + at;
+  if (at >= count) return;
   const int n = g.n, s0 = blockIdx.y * NS;
   ProjSink<NS> sink{xt + (size_t)blockIdx.y * n * n * NS, {}};
-  const FxRay f = rays[ray];
+  FxRay f;
+  if (rays)
+    f = rays[at];
+  else
+    f.nx = kFxExact;
   if (f.nx == kFxExact) {
     Ray r;
     if (setup_row(g, (int32_t)ray, r)) trace(r, sink);
@@ -1769,34 +1775,57 @@ xct_status matfree_project(const Plan& p, const double* cs_dev, const float* x, 
   const int bits = 60 - k;
   const double least = std::min(g.min_seg * (double)(1ll << bits), (double)(1ll << 62));
   const long long min_len = std::max(1ll, (long long)std::llround(least));
+  // Working memory is bounded, and none of it is needed: the rays' walks are
+  // set up for a batch of rays at a time and the slices interleaved for some
+  // tiles at a time; without room for the walks, rays are traced in FP64, and
+  // without room for one tile, slices are read where they are, one a walk.
+  constexpr int64_t kRayBatch = 1 << 22;
+  constexpr size_t kTileBytes = 1ull << 30;
+  const KeepOctets others;
   Arena tmp(s);
-  FxRay* rays;
-  XCT_TRY(tmp.get(&rays, p.nray));
-  fx_setup_kernel<<<grid_for(p.nray, 128), 128, 0, s>>>(gd, p.nray, bits, rays);
-  count_launch();
+  FxRay* rays = nullptr;
+  const int64_t batch = std::min(p.nray, kRayBatch);
+  if (tmp.get(&rays, (size_t)batch) != XCT_OK) rays = nullptr;
   auto run = [&](auto ns) -> xct_status {
     constexpr int NS = decltype(ns)::value;
     const int tiles = (S + NS - 1) / NS;
-    const float* xt = x;
-    if (NS > 1) {
-      float* t;
-      XCT_TRY(tmp.get(&t, (size_t)p.npix * tiles * NS));
-      for (int t0 = 0; t0 < tiles; t0 += 65535)
-        interleave_kernel<NS><<<dim3(grid_for(p.npix, 256), std::min(tiles - t0, 65535)), 256, 0, s>>>(
-            x + (size_t)t0 * NS * p.npix, t + (size_t)t0 * NS * p.npix, p.npix, S - t0 * NS);
-      xt = t;
+    const size_t tile = (size_t)p.npix * NS;
+    const int most = (int)std::min<size_t>(std::max<size_t>(kTileBytes / (tile * sizeof(float)), 1), 65535);
+    const int pass = NS > 1 ? std::min(tiles, most) : std::min(tiles, 65535);
+    float* t = nullptr;
+    if (NS > 1) XCT_TRY(tmp.get(&t, tile * pass));
+    for (int64_t r0 = 0; r0 < p.nray; r0 += batch) {
+      const int64_t nr = std::min(batch, p.nray - r0);
+      if (rays) {
+        fx_setup_kernel<<<grid_for(nr, 128), 128, 0, s>>>(gd, r0, nr, bits, rays);
+        count_launch();
+      }
+      for (int t0 = 0; t0 < tiles; t0 += pass) {
+        const int nt = std::min(tiles - t0, pass);
+        const float* xt = x + (size_t)t0 * tile;
+        if (NS > 1) {
+          if (r0 == 0 || pass < tiles) {
+            interleave_kernel<NS><<<dim3(grid_for(p.npix, 256), nt), 256, 0, s>>>(xt, t, p.npix, S - t0 * NS);
+            count_launch();
+          }
+          xt = t;
+        }
+        matfree_project_kernel<NS><<<dim3(grid_for(nr, 128), nt), 128, 0, s>>>(
+            gd, rays, bits, min_len, xt, y + (size_t)t0 * NS * p.nray, S - t0 * NS, r0, nr, p.nray);
+        count_launch();
+        XCT_TRY_CUDA(cudaGetLastError());
+      }
     }
-    for (int t0 = 0; t0 < tiles; t0 += 65535)
-      matfree_project_kernel<NS><<<dim3(grid_for(p.nray, 128), std::min(tiles - t0, 65535)), 128, 0, s>>>(
-          gd, rays, bits, min_len, xt + (size_t)t0 * NS * p.npix, y + (size_t)t0 * NS * p.nray, S - t0 * NS, p.nray);
-    count_launch(NS > 1 ? 2 : 1);
-    XCT_TRY_CUDA(cudaGetLastError());
     return XCT_OK;
   };
-  if (S == 1) return run(std::integral_constant<int, 1>());
-  if (S == 2) return run(std::integral_constant<int, 2>());
-  if (S <= 4) return run(std::integral_constant<int, 4>());
-  return run(std::integral_constant<int, kMfSlices>());
+  auto tiled = [&]() -> xct_status {
+    if (S == 1) return XCT_ERR_OOM;
+    if (S == 2) return run(std::integral_constant<int, 2>());
+    if (S <= 4) return run(std::integral_constant<int, 4>());
+    return run(std::integral_constant<int, kMfSlices>());
+  };
+  const xct_status st = tiled();
+  return st == XCT_ERR_OOM ? run(std::integral_constant<int, 1>()) : st;
 }
 
 xct_status build_plan(Plan& p, cudaStream_t s) {
