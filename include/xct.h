@@ -158,11 +158,11 @@ typedef struct xct_plan_s* xct_plan_t;
  * 1.42 + 1.35; 1536^2 x 1024: 32.0 + 21.5 beside 20.2 + 17.7).  Where device memory runs out while one is built, or its stages
  * do not fit the product kernel, the plan does without it, and products of
  * that matrix run on the row layouts: slower, and summed in another order
- * (xct_stats tells which are there).  A later allocation of the library that
- * fails takes the octet layouts of all plans of the device on which no product
- * is being enqueued, and is tried again (not those that a captured graph
- * refers to, and not with a caller's allocator; XCT_PLAN_ROWS_ONLY builds
- * none).
+ * (xct_stats tells which are there).  Working memory of a later call that
+ * cannot be had takes the octet layouts of all plans of the device on which no
+ * product is being enqueued, and is asked for again (not those that a captured
+ * graph refers to, and not with a caller's allocator).  The build of another
+ * plan does not take them; XCT_PLAN_ROWS_ONLY builds none.
  * Synchronous: returns when the plan is ready (the work runs on `stream`).
  * `out` receives the plan; on error *out is NULL and nothing is leaked.
  */
@@ -453,12 +453,12 @@ xct_status xct_plan_order(xct_plan_t plan, int32_t* pix, int32_t* ray);
  * from a pool of the library's own, which holds up to 4 GiB of it mapped between
  * calls.  That memory goes back to the device when the last plan is released
  * and whenever an allocation of the library fails, which is then tried once
- * more, at last without the octet layouts of plans (see xct_plan; not under
- * stream capture).  A caller may route every allocation
- * through its own allocator (e.g. a framework's caching allocator); the
- * callbacks must be thread-safe and remain valid until reset.  alloc returns
- * NULL on failure (the library then returns XCT_ERR_OOM and frees what it
- * took).  Passing NULL, NULL restores the default.
+ * more (a call's working memory at last without the octet layouts of plans,
+ * see xct_plan; not under stream capture).  A caller may route every
+ * allocation through its own allocator (e.g. a framework's caching allocator);
+ * the callbacks must be thread-safe and remain valid until reset.  alloc
+ * returns NULL on failure (the library then returns XCT_ERR_OOM and frees what
+ * it took).  Passing NULL, NULL restores the default.
  */
 typedef void* (*xct_alloc_fn)(size_t bytes, void* stream, void* ctx);
 typedef void (*xct_free_fn)(void* ptr, size_t bytes, void* stream, void* ctx);

@@ -779,6 +779,9 @@ xct_status xct_plan(const xct_geometry* g, xct_dtype storage, uint32_t flags, vo
     return XCT_ERR_CUDA;
   }
   scratch_plans(p->device, 1);
+  // (another plan's products do not become slower for this one: it is built
+  // with what memory there is, or not)
+  const KeepOctets others;
   xct_status st = build_plan(*p, s);
   if (st != XCT_OK) {
     cudaStreamSynchronize(s);

@@ -1979,7 +1979,6 @@ xct_status build_plan(Plan& p, cudaStream_t s) {
   // where device memory runs out or a stage does not fit, those products use
   // the layouts above
   if (stages16(p.storage) && !(p.flags & XCT_PLAN_ROWS_ONLY)) {
-    const KeepOctets others;
     p.oct_mem.stream = s;
     for (int which = 0; which < 2; ++which) {
       Arena mem(s, true);
