@@ -184,11 +184,14 @@ xct_status xct_project(xct_plan_t plan, const float* x, float* y, int32_t S,
 
 /*
  * xct_project_rows -- xct_project with every ray's sum taken in the order of
- * its stored entries, as the products inside xct_cgls take it (xct_project
- * and xct_backproject of 16-bit slices sum blocks of 16 columns on the
- * tensor cores first: the same FP32 accumulation in another order).  For
- * costs that are reported in FP64: the data term of the differentiable
- * reconstruction is computed from it.
+ * its stored entries, every addition rounded to nearest, as the products
+ * inside xct_cgls take it.  (xct_project and xct_backproject of 16-bit slices
+ * sum pieces of 16 columns on the tensor cores, which cut what lies below
+ * about 2^-24 of the largest term, and add the pieces in FP32 to nearest: their
+ * error against 64 bits is no larger than the row order's, but binary16 sums
+ * of positive terms come out about 2e-8 low on average.)  For costs that are
+ * reported in FP64: the data term of the differentiable reconstruction is
+ * computed from it.
  */
 xct_status xct_project_rows(xct_plan_t plan, const float* x, float* y, int32_t S,
                             void* stream);

@@ -40,7 +40,10 @@ namespace {
 constexpr int kMmaWarps = kOcts;                 // consumer warps
 constexpr int kMaxBufs = 4;                      // stage buffers, a copy warp for each
 constexpr int kSlots = 2 * kMaxBufs;             // stage descriptors in flight
-constexpr int kMmaThreads = (kMmaWarps + 1 + kMaxBufs) * 32;
+// of a tile width: with 32 and 64 slices no more than 3 fit (2 with 64 on a
+// large grid), and 20 warps may use 96 registers where 21 may use 80
+constexpr int max_bufs(int st) { return st >= 32 ? 3 : kMaxBufs; }
+constexpr int mma_threads(int st) { return (kMmaWarps + 1 + max_bufs(st)) * 32; }
 constexpr size_t kMmaSmem = 227 * 1024;          // of one CTA per SM
 constexpr uint32_t kHdrBytes = 16 * kMmaWarps;   // stage header: 16 bytes for every consumer warp
 constexpr uint32_t kFirst = 1, kLast = 2, kEnd = 4, kReal = 8;   // of its block; no more work; has entries
@@ -117,9 +120,39 @@ __device__ __forceinline__ void add2(float* acc, const float* d) {
   acc[0] = s.x;
   acc[1] = s.y;
 }
+// sum = or += a chunk times MT * 16 slices
+template <bool FIRST, class TX, int MT>
+__device__ __forceinline__ void chunk_times(float (&sum)[MT][4], const uint32_t (&x)[MT][4], uint2 w) {
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    if constexpr (FIRST) {
+      mma_16816(sum[i], x[i], w, TX());
+    } else {
+      float d[4];
+      mma_16816(d, x[i], w, TX());
+      add2(sum[i], d);
+      add2(sum[i] + 2, d + 2);
+    }
+  }
+}
+// to += what
+template <int MT>
+__device__ __forceinline__ void add_sums(float (&to)[MT][4], const float (&what)[MT][4]) {
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    add2(to[i], what[i]);
+    add2(to[i] + 2, what[i] + 2);
+  }
+}
+// acc + low += d, low taking what acc's rounding loses (two-sum, Knuth)
+__device__ __forceinline__ void add_exact(float& acc, float& low, float d) {
+  const float s = __fadd_rn(acc, d), v = __fsub_rn(s, acc);
+  low = __fadd_rn(low, __fadd_rn(__fsub_rn(acc, __fsub_rn(s, v)), __fsub_rn(d, v)));
+  acc = s;
+}
 
 template <class TX, int ST>
-__global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
+__global__ void __launch_bounds__(mma_threads(ST), 1) spmm_mma_kernel(MmaArgs a) {
   constexpr int ROWB = 2 * ST;                        // bytes of a staged row
   constexpr int MT = ST < 16 ? 1 : ST / 16;           // MMAs per chunk
   constexpr int HN = ST < 16 ? 1 : 2;                 // 8-slice halves of an MMA's rows in use
@@ -288,8 +321,21 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
   // 8-slice half it reads of it
   const int lk = ST < 16 ? (lane & 15) : (lane & 7) + ((lane >> 4) << 3);
   const uint32_t lh = ST < 16 ? 0u : (uint32_t)(lane >> 3) & 1u;
-  float acc[MT][4];
-  float scale[MT * HN];
+  // A row's 50 to 150 chunks added one after the other err more than the row
+  // layouts, whose rows several lanes share, with 8 and 64 slices.  There the
+  // chunks of a stage are summed first, then the stages: for 8 slices with
+  // what their rounding loses, for 64 bfloat16 ones into two sums in turn.
+  // Error of sums of positive terms at 400^2 x 300, in 10^-9 of the sum (rms;
+  // rows, one level, as here): 8 slices binary16 86, 162, 34, bfloat16 45, 138,
+  // 27; 64 slices 159, 162, 70 and 74, 138, 47; 16 and 32 slices, in one level,
+  // 306, 162 and 177, 138.  512^2 x 768: 8 slices 0.308 -> 0.311 ms, 64 slices
+  // binary16 0.685 -> 0.680, bfloat16 0.685 -> 0.704 (scales formed at a
+  // block's end, out of the loop's registers: 64 slices 0.697 -> 0.680).
+  constexpr bool EXACT = ST == 8, TWO = ST == 64;
+  constexpr int NA = TWO && std::is_same<TX, __nv_bfloat16>::value ? 2 : 1;
+  float acc[NA][MT][4];
+  float low[EXACT ? 4 : 1];
+  bool second = false;   // the sum that takes the next stage
   bool finite = true;
   int buf = 0;
   uint32_t use = 0;
@@ -303,6 +349,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
     if (word.w & kFirst) {
       const uint32_t* im = a.in_max + (word.z / (uint32_t)a.nblocks) * ST;
       uint32_t big = 0;
+      second = false;
 #pragma unroll
       for (int i = 0; i < MT; ++i)
 #pragma unroll
@@ -310,13 +357,17 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
           const uint32_t mb = __ldg(im + 16 * i + 8 * q + g);
           // (or is so small, at most 2^-128, that its scale is infinite)
           big |= mb >= 0x7f800000u || mb - 1u < 0x00200000u;
-          scale[i * HN + q] = ldexpf(1.0f, ceil_log2_exp_p(__uint_as_float(mb)) - a.mat_scale_exp);
         }
       finite = !__any_sync(0xffffffffu, big != 0u);
 #pragma unroll
       for (int i = 0; i < MT; ++i)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[i][q] = 0.0f;
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+          for (int k = 0; k < NA; ++k) acc[k][i][q] = 0.0f;
+      if constexpr (EXACT)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) low[q] = 0.0f;
     }
     if (word.x & 0xffffu) {
       const int c0 = (int)(word.x >> 16), n = (int)(word.x & 0xffffu);
@@ -327,6 +378,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
         return xb + pos * ROWB + ((lh ^ ((pos >> SH) & MASK)) << 4);
       };
       if (finite) {
+        float own[MT][4] = {};
+        float (&part)[MT][4] = EXACT || TWO ? own : acc[0];   // takes the stage's chunks
         uint32_t pa = pb + c0 * 32 + lk * 2, wa = eb + c0 * 256 + lane * 8;
         auto gather = [&](uint32_t (&x)[MT][4], uint32_t pos) {
           const uint32_t ad = row_addr(pos);
@@ -336,15 +389,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
           } else {
             ldsm_x2_t(x[0][0], x[0][2], ad);
             x[0][1] = x[0][3] = 0u;
-          }
-        };
-        auto multiply = [&](const uint32_t (&x)[MT][4], uint2 w) {
-#pragma unroll
-          for (int i = 0; i < MT; ++i) {
-            float d[4];
-            mma_16816(d, x[i], w, TX());
-            add2(acc[i], d);
-            add2(acc[i] + 2, d + 2);
           }
         };
         // U chunks at a time, the next U chunks' positions and values loaded
@@ -366,6 +410,13 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
         };
         fetch(n);
         int left = n;
+        if constexpr (TWO) {   // the first chunk: no sum to add it to
+          uint32_t x[MT][4];
+          gather(x, p[0]);
+          const uint2 wc = w[0];
+          fetch(--left);
+          chunk_times<true, TX>(part, x, wc);
+        }
         for (; left >= U; left -= U) {
           uint32_t x[U][MT][4];
           uint2 wc[U];
@@ -376,15 +427,25 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
           }
           fetch(left - U);
 #pragma unroll
-          for (int u = 0; u < U; ++u) multiply(x[u], wc[u]);
+          for (int u = 0; u < U; ++u) chunk_times<false, TX>(part, x[u], wc[u]);
         }
 #pragma unroll
         for (int u = 0; u < U - 1; ++u)
           if (u < left) {
             uint32_t x[MT][4];
             gather(x, p[u]);
-            multiply(x, w[u]);
+            chunk_times<false, TX>(part, x, w[u]);
           }
+        if constexpr (EXACT) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) add_exact(acc[0][0][q], low[q], part[0][q]);
+        } else if constexpr (TWO) {
+          if (NA > 1 && second)
+            add_sums(acc[NA - 1], part);
+          else
+            add_sums(acc[0], part);
+          second = !second;
+        }
       } else {
         // a slice of this tile is staged with infinities or NaN: 0 times it in a
         // chunk's unused cells would reach rows that do not cross it, so the
@@ -400,8 +461,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
               for (int q = 0; q < HN; ++q) {
                 const float xv = to_f32(
                     lds_u16(xb + pos * ROWB + (((uint32_t)(2 * i + q) ^ ((pos >> SH) & MASK)) << 4) + g * 2), TX());
-                if (w0 & 0x7fffu) acc[i][2 * q] = fmaf(to_f32(w0, TX()), xv, acc[i][2 * q]);
-                if (w1 & 0x7fffu) acc[i][2 * q + 1] = fmaf(to_f32(w1, TX()), xv, acc[i][2 * q + 1]);
+                if (w0 & 0x7fffu) acc[0][i][2 * q] = fmaf(to_f32(w0, TX()), xv, acc[0][i][2 * q]);
+                if (w1 & 0x7fffu) acc[0][i][2 * q + 1] = fmaf(to_f32(w1, TX()), xv, acc[0][i][2 * q + 1]);
               }
           }
       }
@@ -409,6 +470,12 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[buf]);
     if (word.w & kLast) {
+      if constexpr (EXACT) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[0][0][q] += low[q];
+      } else if constexpr (NA > 1) {
+        add_sums(acc[0], acc[NA - 1]);
+      }
       // ---- epilogue of a block: de-normalise, write to the natural layout
       // (the lane's two rows are neighbouring bins or pixels of a full tile)
       const int tile = (int)(word.z / (uint32_t)a.nblocks), b = (int)(word.z % (uint32_t)a.nblocks);
@@ -425,7 +492,9 @@ __global__ void __launch_bounds__(kMmaThreads, 1) spmm_mma_kernel(MmaArgs a) {
           const int sl = tile * ST + 16 * i + 8 * q + g;
           if (sl >= a.S) continue;
           float* dst = a.y + (size_t)sl * a.nrows;
-          const float u = acc[i][2 * q] * scale[i * HN + q], v = acc[i][2 * q + 1] * scale[i * HN + q];
+          const uint32_t mb = __ldg(a.in_max + tile * ST + 16 * i + 8 * q + g);
+          const float scale = ldexpf(1.0f, ceil_log2_exp_p(__uint_as_float(mb)) - a.mat_scale_exp);
+          const float u = acc[0][i][2 * q] * scale, v = acc[0][i][2 * q + 1] * scale;
           if (two) {
             *reinterpret_cast<float2*>(dst + n0) = make_float2(u, v);
           } else {
@@ -448,12 +517,12 @@ size_t fixed_smem(size_t dbytes) {
   return kSlots * dbytes + 8 * (2 * kMaxBufs + 2 * kSlots) + 8 * kSlots + 128;
 }
 
-// stage buffers that fit a CTA, at most kMaxBufs
-int buffers(size_t xbytes, size_t ebytes, size_t dbytes) {
+// stage buffers that fit a CTA, at most `most`
+int buffers(size_t xbytes, size_t ebytes, size_t dbytes, int most) {
   const size_t fixed = fixed_smem(dbytes);
   if (fixed >= kMmaSmem) return 0;
   const size_t n = (kMmaSmem - fixed) / (xbytes + ebytes + kHdrBytes);
-  return n < (size_t)kMaxBufs ? (int)n : kMaxBufs;
+  return n < (size_t)most ? (int)n : most;
 }
 
 // ---------------------------------------------------------------------------
@@ -574,7 +643,7 @@ xct_status launch_mma(const OctLayout& L, const OctProduct& p, cudaStream_t st) 
   a.xbytes = (uint32_t)align128((size_t)L.cap * 2 * ST);
   a.ebytes = (uint32_t)align128((size_t)L.emax * kChunkBytes);
   a.dbytes = (uint32_t)align128((size_t)L.desc_bytes);
-  a.nbufs = buffers(a.xbytes, a.ebytes, a.dbytes);
+  a.nbufs = buffers(a.xbytes, a.ebytes, a.dbytes, max_bufs(ST));
   const size_t smem = fixed_smem(a.dbytes) + a.nbufs * (size_t)(a.xbytes + a.ebytes + kHdrBytes);
   int dev = 0, sms = 0;
   XCT_TRY_CUDA(cudaGetDevice(&dev));
@@ -585,7 +654,7 @@ xct_status launch_mma(const OctLayout& L, const OctProduct& p, cudaStream_t st) 
                                       (int)kMmaSmem));
     if (dev >= 0 && dev < kMaxDevices) configured[dev].store(true);
   }
-  spmm_mma_kernel<TX, ST><<<a.nwork < sms ? a.nwork : sms, kMmaThreads, smem, st>>>(a);
+  spmm_mma_kernel<TX, ST><<<a.nwork < sms ? a.nwork : sms, mma_threads(ST), smem, st>>>(a);
   count_launch();
   XCT_TRY_CUDA(cudaGetLastError());
   return XCT_OK;
@@ -612,7 +681,7 @@ xct_status by_tile(xct_dtype storage, int st, F f) {
 }  // namespace
 
 bool oct_stage_fits(int cap, int64_t emax, int64_t desc_bytes) {
-  return buffers(align128((size_t)cap * 128), align128((size_t)emax * kChunkBytes), align128((size_t)desc_bytes)) >= 2;
+  return buffers(align128((size_t)cap * 128), align128((size_t)emax * kChunkBytes), align128((size_t)desc_bytes), 2) >= 2;
 }
 
 xct_status oct_stage(const OctLayout& L, const OctProduct& p, xct_dtype storage, cudaStream_t s) {
