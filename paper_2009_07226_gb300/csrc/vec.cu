@@ -29,7 +29,7 @@ template <int ST>
 __global__ void __launch_bounds__(kConvThreads) to_internal_kernel(
     const float* __restrict__ nat, float* __restrict__ out, const int32_t* __restrict__ inv,
     int64_t rows, int S, uint32_t* __restrict__ max_bits) {
-  constexpr int R = conv_rows(ST), V = ST >= 4 ? 4 : ST;
+  constexpr int R = conv_rows(ST), V = 4;
   __shared__ float buf[ST][R + 1];
   __shared__ uint32_t smax[ST];
   const int64_t h0 = (int64_t)blockIdx.x * R;
@@ -55,12 +55,7 @@ __global__ void __launch_bounds__(kConvThreads) to_internal_kernel(
   float* dst = out + ((size_t)t * rows + h0) * ST;
   for (int i = threadIdx.x; i < nr * (ST / V); i += kConvThreads) {
     const int row = i / (ST / V), sl = i % (ST / V) * V;
-    if constexpr (V == 4) {
-      reinterpret_cast<float4*>(dst)[i] = make_float4(buf[sl][row], buf[sl + 1][row], buf[sl + 2][row], buf[sl + 3][row]);
-    } else {
-#pragma unroll
-      for (int v = 0; v < V; ++v) dst[i * V + v] = buf[sl + v][row];
-    }
+    reinterpret_cast<float4*>(dst)[i] = make_float4(buf[sl][row], buf[sl + 1][row], buf[sl + 2][row], buf[sl + 3][row]);
   }
   if (max_bits && threadIdx.x < ST) {
     const uint32_t m = smax[threadIdx.x];
@@ -73,7 +68,7 @@ template <int ST>
 __global__ void __launch_bounds__(kConvThreads) to_natural_kernel(
     const float* __restrict__ in, float* __restrict__ nat, const int32_t* __restrict__ inv,
     int64_t rows, int S) {
-  constexpr int R = conv_rows(ST), V = ST >= 4 ? 4 : ST;
+  constexpr int R = conv_rows(ST), V = 4;
   __shared__ float buf[ST][R + 1];
   const int64_t h0 = (int64_t)blockIdx.x * R;
   const int t = blockIdx.y, live = min(ST, S - t * ST);
@@ -86,16 +81,11 @@ __global__ void __launch_bounds__(kConvThreads) to_natural_kernel(
   for (int i = threadIdx.x; i < nr * (ST / V); i += kConvThreads) {
     const int row = i / (ST / V), sl = i % (ST / V) * V;
     if (sl >= live) continue;
-    if constexpr (V == 4) {
-      const float4 v = reinterpret_cast<const float4*>(src)[i];
-      buf[sl][row] = v.x;
-      buf[sl + 1][row] = v.y;
-      buf[sl + 2][row] = v.z;
-      buf[sl + 3][row] = v.w;
-    } else {
-#pragma unroll
-      for (int v = 0; v < V; ++v) buf[sl + v][row] = src[i * V + v];
-    }
+    const float4 v = reinterpret_cast<const float4*>(src)[i];
+    buf[sl][row] = v.x;
+    buf[sl + 1][row] = v.y;
+    buf[sl + 2][row] = v.z;
+    buf[sl + 3][row] = v.w;
   }
   __syncthreads();
   const int r = threadIdx.x % R;
@@ -526,12 +516,10 @@ __global__ void cgls_save_kernel(const CglsScalars sc, int S, CglsStateHeader hd
   if (threadIdx.x == 0) *hdr_out = hdr;
 }
 
-// f(integral constant of the tile width)
+// f(integral constant of the tile width; pick_slices_per_tile gives none below 4)
 template <class F>
 xct_status by_width(int st, F f) {
   switch (st) {
-    case 1: XCT_TRY_CUDA(f(std::integral_constant<int, 1>())); break;
-    case 2: XCT_TRY_CUDA(f(std::integral_constant<int, 2>())); break;
     case 4: XCT_TRY_CUDA(f(std::integral_constant<int, 4>())); break;
     case 8: XCT_TRY_CUDA(f(std::integral_constant<int, 8>())); break;
     case 16: XCT_TRY_CUDA(f(std::integral_constant<int, 16>())); break;
