@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(PCfg<TX, TW, ST>::NT, PCfg<TX, TW, ST>::MINB)
       }
     };
     bool ok = true;
-    uint32_t end_it = 0, req_hi = 0;   // first stage not filled; last one whose descriptor was requested
+    uint32_t fail_it = 0, req_hi = 0;   // req_hi: last stage whose descriptor was requested
     for (int j = 0; j < kDescAhead; ++j) {
       request(cur, j);
       advance(cur);
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(PCfg<TX, TW, ST>::NT, PCfg<TX, TW, ST>::MINB)
       request(cur, (int)((it + kDescAhead) % DS));
       req_hi = it + kDescAhead;
       advance(cur);
-      if (!mbar_wait(&dbar[ds], (it / DS) & 1, a.wait_ns)) { ok = false; end_it = it; break; }
+      if (!mbar_wait(&dbar[ds], (it / DS) & 1, a.wait_ns)) { ok = false; fail_it = it; break; }
       __syncwarp();
       const int4 id = ident[ds];
       const bool real = (id.w & 2) != 0;
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(PCfg<TX, TW, ST>::NT, PCfg<TX, TW, ST>::MINB)
       // about two stages from now, are brought into L2 before this warp
       // waits for the buffer (measured 3.5% faster than no prefetch)
       if (WIDE && lane == 0 && eb) bulk_prefetch_l2(P.ent + (size_t)dh.e0 * EB, eb);
-      if (!mbar_wait(&empty[buf], (use & 1) ^ 1, a.wait_ns)) { ok = false; end_it = it; break; }
+      if (!mbar_wait(&empty[buf], (use & 1) ^ 1, a.wait_ns)) { ok = false; fail_it = it; break; }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       if (lane == 0) {
         Hdr h;
@@ -429,19 +429,26 @@ __global__ void __launch_bounds__(PCfg<TX, TW, ST>::NT, PCfg<TX, TW, ST>::MINB)
       // the single arrival of this phase; it also publishes the header
       __syncwarp();
       if (lane == 0) mbar_arrive(&full[buf]);
-      if (id.x < 0) { end_it = it + 1; break; }
+      if (id.x < 0) {
+        // the last stages' copies land, too: consumers that gave up do not
+        // wait for them (no descriptor is under way: those past the last
+        // stage are requested without a copy)
+        for (uint32_t j = it > (uint32_t)NB - 1 ? it - (NB - 1) : 0; j < it; ++j)
+          mbar_wait(&full[j % NB], (j / NB) & 1, kDrainNs);
+        break;
+      }
     }
-    // Copies already issued land before the CTA's shared memory goes away,
-    // after the last stage too (consumers that gave up do not wait for them):
-    // the stage copies of the last NB iterations that arrived on their full
-    // barrier (every one before end_it did, with copies or without), and the
-    // descriptors requested for stages end_it to req_hi (every request
-    // completes a phase of its slot's barrier; past the last stage without a
-    // copy).
-    if (!ok && lane == 0) atomicExch(a.err, 1);
-    for (uint32_t j = end_it > (uint32_t)NB ? end_it - NB : 0; j < end_it; ++j)
-      mbar_wait(&full[j % NB], (j / NB) & 1, kDrainNs);
-    for (uint32_t j = end_it; j <= req_hi; ++j) mbar_wait(&dbar[j % DS], (j / DS) & 1, kDrainNs);
+    if (!ok) {
+      if (lane == 0) atomicExch(a.err, 1);
+      // let copies already issued land before the CTA's shared memory goes
+      // away: the stage copies of the last NB iterations before the failing
+      // one (every iteration arrives on its full barrier, with copies or
+      // without), and the descriptors requested for stages fail_it to req_hi
+      // (every request completes a phase of its slot's barrier)
+      for (uint32_t j = fail_it > (uint32_t)NB ? fail_it - NB : 0; j < fail_it; ++j)
+        mbar_wait(&full[j % NB], (j / NB) & 1, kDrainNs);
+      for (uint32_t j = fail_it; j <= req_hi; ++j) mbar_wait(&dbar[j % DS], (j / DS) & 1, kDrainNs);
+    }
     return;
   }
 
