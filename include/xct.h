@@ -258,8 +258,7 @@ xct_status xct_cgls_matfree(xct_plan_t plan, const float* y, float* x, int32_t S
  * FP64 CGLS scalars.  x: [S][n][n] float64, y: [S][n_angles][n_det] float64
  * (natural layouts as above), host or device.  xct_cgls_f64 runs the
  * recurrence of xct_cgls (flags: XCT_CGLS_X0 only; resid as there; the same
- * stop and XCT_ERR_BREAKDOWN rules) with launches issued directly (no
- * graph), and returns when the solve is done.  The products are bound by
+ * stop and XCT_ERR_BREAKDOWN rules) and returns when the solve is done.  The products are bound by
  * the GPU's FP64 FMA rate.
  */
 xct_status xct_project_f64(xct_plan_t plan, const double* x, double* y, int32_t S,

@@ -337,7 +337,7 @@ xct_status spmm_timed(const SpmmArgs& a, int kind, PhaseTimer* tm, cudaStream_t 
   return XCT_OK;
 }
 
-// Enqueue the whole solve on stream s (graph-capturable: no host syncs).
+// Enqueue the whole solve on stream s (no host syncs).
 xct_status enqueue_cgls(Plan& p, const float* yd, float* xd, int S, int st, int ntiles, int iters,
                         bool x0, CglsBufs& B, cudaStream_t s, PhaseTimer* tm,
                         const CglsState* resume = nullptr, const CglsState* save = nullptr,

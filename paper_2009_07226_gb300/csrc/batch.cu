@@ -286,8 +286,9 @@ extern "C" xct_status xct_cgls_batch(const xct_job* jobs, int32_t n_jobs, int32_
   XCT_TRY(ar.get(&work, 1));
   const bool x0 = (flags & XCT_CGLS_X0) != 0;
   // launched directly: capturing and instantiating a graph that runs once
-  // costs more than its launches (four jobs of up to 384^2, 3 iterations: 4.90
-  // against 4.65 ms)
+  // costs more than its launches (four jobs of up to 384^2: 3 iterations 5.63
+  // against 5.38 ms, 20 27.5 against 26.6, 50 66.0 against 64.0; xct_cgls of a
+  // 128^2 slice: 5 iterations 0.83 against 0.72 ms, 50 5.99 against 5.50)
   XCT_TRY(enqueue_batch(G, jobs, iters, x0, work, us));
   // per-job residual logs: the job's slices of the group log
   for (auto& g : G)

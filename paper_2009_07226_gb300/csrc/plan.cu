@@ -352,9 +352,9 @@ __global__ void siddon_fill_kernel(GeomDev g, const int32_t* ray_inv, const int3
 // that are not unit vectors are traced as the plan builder traces them.
 // The slices are interleaved in tiles first, so a step reads one contiguous
 // piece of kMfSlices slices instead of as many distant words.
-// 256^2 x 384, 24 slices: 61.7 -> 0.73 ms a call (three tiles of 8; before,
+// 256^2 x 384, 24 slices: 61.7 -> 0.74 ms a call (three tiles of 8; before,
 // every tile walked in FP64 and read each slice on its own); steps of whole
-// units would take 0.72.
+// units would take 0.73.
 constexpr int kMfSlices = 8;
 
 struct FxRay {

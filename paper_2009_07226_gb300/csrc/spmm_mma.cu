@@ -7,7 +7,7 @@
 // MMA's rows, the octet's rows as its columns, FP32 accumulators.  The staged
 // rows that a chunk names are gathered from shared memory by ldmatrix with
 // transposition, 8 arbitrary rows per phase; row chunks are permuted by the
-// row's id (to_staged16_kernel) and the plan gives a phase's rows distinct
+// row's id (stage_natural_kernel) and the plan gives a phase's rows distinct
 // ids mod 8, so a phase is conflict-free.
 //
 // A persistent CTA per SM: a scheduler warp walks the stages and requests
@@ -16,17 +16,18 @@
 // 16 consumer warps take one octet each and write its rows in the caller's
 // layout.
 //
-// What bounds it (512^2 x 768 x 512, binary16): with 64 slices the shared-memory
-// data path (16 wavefronts a chunk for the gathers, 3 for values and
-// positions and 3 of conflicts, plus the copies' writes): 0.69 ms per
-// xct_project, 0.65 per xct_backproject, 0.05 to 0.07 of them staging, against
-// 1.45 / 1.41 on the paired row layouts (spmm_pipe.cu) with their conversions;
-// 32 slices 0.41 / 0.38, 16 slices 0.33 / 0.32 and 8 slices 0.31 / 0.30 (the
-// FMA kernels alone 0.77 / 0.76, 0.49 / 0.50 and 0.45 / 0.43), there close to
-// the chunks' stream from device memory (1.8 GB, 0.26 ms).  At 1536^2 x 1024
-// the blocks' copies come from L2 at about 9 TB/s, its bound there.  tcgen05
-// would want 64 or more rows an operand tile, where only a tenth of the cells
-// are entries: more bytes from device memory than the sparse form needs.
+// What bounds it (512^2 x 768 x 512, binary16): with 64 slices shared memory,
+// where a chunk's 16 gathered rows (2048 bytes) and its values and positions
+// (288) take 19 wavefronts of 128 bytes, 0.37 ms of the product for its 6.2 M
+// chunks, and the copies write the stages: 0.68 ms per xct_project, 0.65 per
+// xct_backproject, 0.05 to 0.07 of them staging, against 1.45 / 1.41 on the
+// paired row layouts (spmm_pipe.cu) with their conversions; 32 slices 0.40 /
+// 0.38, 16 slices 0.33 / 0.32 and 8 slices 0.31 / 0.30 (the FMA kernels alone
+// 0.77 / 0.76, 0.49 / 0.50 and 0.45 / 0.43), there close to the chunks' stream
+// from device memory (1.8 GB, 0.27 ms).  At 1536^2 x 1024, 32 slices, the
+// stream of 32 GB takes 4.8 ms of the 5.8 at the measured copy bandwidth.
+// tcgen05 would want 64 or more rows an operand tile, where only a tenth of the
+// cells are entries: more bytes from device memory than the sparse form needs.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
