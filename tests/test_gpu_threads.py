@@ -55,3 +55,26 @@ def test_plans_of_different_sizes_built_at_once(xct, kind):
     for t in threads:
         t.join()
     assert not errors, errors[:4]
+
+
+def test_many_small_and_large_plans_built_at_once(xct):
+    """Eight threads, 4400 builds: a block's footprint needs 1 KB of shared
+    memory in some and over 100 KB in the others, rays 8 pixels apart."""
+    errors = []
+
+    def work(n, m, nd, spacing, builds):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(builds):
+                try:
+                    with xct.Plan(n, m, nd, "f16", cos_sin=inputs.angle_table(m), det_spacing=spacing):
+                        pass
+                except xct.XctError as e:
+                    errors.append(str(e))
+
+    threads = [threading.Thread(target=work, args=a)
+               for a in [(12, 10, 12, 1.0, 800)] * 4 + [(360, 16, 45, 8.0, 300)] * 4]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, (len(errors), errors[:2])
